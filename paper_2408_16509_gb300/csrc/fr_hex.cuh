@@ -137,7 +137,12 @@ __device__ __forceinline__ void hex_stage_apply(const HexStage<T, TR>& a,
                                                 T s[5]) {
   bool bad = false;
 #pragma unroll
-  for (int k = 0; k < 5; ++k) bad |= !isfinite(R[k]);
+  for (int k = 0; k < 5; ++k) {
+    if constexpr (sizeof(T) == 8)  // exponent bits: no FP64 comparison
+      bad |= (__double2hiint(R[k]) & 0x7ff00000) == 0x7ff00000;
+    else
+      bad |= !isfinite(R[k]);
+  }
   if (bad) atomicOr(a.flag, 1);
   if (a.mode == 0) {
 #pragma unroll

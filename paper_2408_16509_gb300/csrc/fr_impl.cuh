@@ -20,9 +20,11 @@
 
 #include "../../include/frgb.h"
 #include "fr_aa.cuh"
+#include "fr_dd.hpp"
 #include "fr_dense_tc.cuh"
 #include "fr_filter.cuh"
 #include "fr_hex.cuh"
+#include "fr_hexfx.cuh"
 #include "fr_kernels.cuh"
 #include "fr_prism.cuh"
 #include "fr_err.hpp"
@@ -91,13 +93,20 @@ struct DevType {
   void* R = nullptr;        // right-hand side (fr_rhs)
   void* smat = nullptr;     // [ne][9][nu]
   void* rcpdjac = nullptr;  // [ne][nu]
-  void* grad = nullptr;     // [ne][15][nu] (NS)
+  void* grad = nullptr;     // [ne][15][nu] (NS); the FP64 fixed-point kernels
+                            // keep the viscous flux in it, [ne][9][nu]
   void* M0T = nullptr;
   void* DT = nullptr;
   void* LIFTT = nullptr;
   void* NREF = nullptr;
   HexOps<double> hx64{};
   HexOps<float> hx32{};
+  // FP64 fixed-point kernels: line operators, S and S / det J in limbs
+  // [ne][9][nu], their exponents [ne][4]
+  HexFxOps hxfx{};
+  FxCoef* fxs = nullptr;
+  FxCoef* fxj = nullptr;
+  int* fxe = nullptr;
   // entropy filter (allocated by fr_filter_enable)
   void* fVinvT = nullptr;
   void* fVT = nullptr;
@@ -436,6 +445,56 @@ HexOps<T> hex_ops(const RefElement& R) {
   return h;
 }
 
+// Line operators of the FP64 fixed-point kernels (fr_hexfx.cuh) in limbs,
+// scaled by powers of two that bound the rows' sums of magnitudes.
+inline HexFxOps hex_fx_ops(const RefElement& R) {
+  HexFxOps o{};
+  const DDLine X = dd_line_ops(R.x1, R.family);
+  const int n = R.p + 1, P = n / 2, H = (n + 1) / 2;
+  auto scale = [](double bound) {  // smallest s >= 1 with bound <= 2^s
+    int s = 1;
+    while (std::ldexp(1.0, s) < bound) ++s;
+    return s;
+  };
+  auto limbs = [](DD x, int s) { return fx_split(dd_fixed(x, s)); };
+  double sl = 0.0, bg = 0.0, bv = 0.0;
+  for (int m = 0; m < n; ++m) sl += std::fabs(X.lm[m].hi);
+  o.sm = scale(sl);
+  const double js = std::ldexp(1.0, o.sm);  // the volume kernel's jump scale
+  for (int a = 0; a < n; ++a) {
+    double d = 0.0;
+    for (int m = 0; m < n; ++m) d += std::fabs(X.d[a * n + m].hi);
+    const double c = std::fabs(X.gr[a].hi) + std::fabs(X.gr[n - 1 - a].hi);
+    bg = std::max(bg, d + c);
+    bv = std::max(bv, d + 1.5 * js * c);  // a jump is below 1.5 of its scale
+  }
+  o.sg = scale(bg);
+  o.sv = scale(bv);
+  auto rows = [&](HexFxLine& L, int s, double jscale) {
+    for (int i = 0; i < H; ++i) {
+      const DD* D = &X.d[size_t(i) * n];
+      const DD gr = X.gr[i], gl = X.gr[n - 1 - i], w(0.5 * jscale);
+      for (int m = 0; m < P; ++m) {
+        L.b[i][m] = limbs(DD(0.5) * (D[m] - D[n - 1 - m]), s);
+        if (i < P) L.a[i][m] = limbs(DD(0.5) * (D[m] + D[n - 1 - m]), s);
+      }
+      L.cb[i] = limbs(-(w * (gl + gr)), s);
+      if (i < P) {
+        if (n % 2) L.a[i][P] = limbs(D[P], s);
+        L.ca[i] = limbs(w * (gr - gl), s);
+      }
+    }
+  };
+  rows(o.g, o.sg, 1.0);
+  rows(o.v, o.sv, js);
+  for (int m = 0; m < P; ++m) {
+    o.ie[m] = limbs(DD(0.5) * (X.lm[m] + X.lm[n - 1 - m]), o.sm);
+    o.io[m] = limbs(DD(0.5) * (X.lm[m] - X.lm[n - 1 - m]), o.sm);
+  }
+  if (n % 2) o.ie[P] = limbs(X.lm[P], o.sm);
+  return o;
+}
+
 // TF32 value of x rounded to nearest, ties away from zero (the rounding of
 // cvt.rna.tf32.f32): the low 13 mantissa bits become zero.
 float tf32_rna_host(float x) {
@@ -659,6 +718,22 @@ int setup_device(fr_mesh* m) {
     if (D.kind == EK_HEX) {
       D.hx64 = hex_ops<double>(R);
       D.hx32 = hex_ops<float>(R);
+      if constexpr (sizeof(T) == 8) {
+        if (m->order >= 2) {
+          D.hxfx = hex_fx_ops(R);
+          const size_t bytes = size_t(D.ne) * 9 * D.nu * sizeof(FxCoef);
+          if ((rc = dev_zeros(m, bytes, (void**)&D.fxs))) return rc;
+          if (m->physics == FR_NAVIER_STOKES && (rc = dev_zeros(m, bytes, (void**)&D.fxj)))
+            return rc;
+          if ((rc = dev_zeros(m, size_t(D.ne) * 4 * sizeof(int), (void**)&D.fxe))) return rc;
+          dispatch(D.kind, m->order, [&](auto nu, auto) {
+            k_fx_metric<decltype(nu)::value><<<unsigned((D.ne * 32 + 255) / 256), 256>>>(
+                D.ne, (const double*)D.smat, (const double*)D.rcpdjac, D.fxs, D.fxj, D.fxe);
+          });
+          CK(cudaGetLastError());
+          CK(cudaDeviceSynchronize());
+        }
+      }
       if (sizeof(T) == 4 && !D.curved) {  // vertex metrics for the FP32-value kernels
         std::vector<double> xv(size_t(D.ne) * 24);
         for (long long e = 0; e < D.ne; ++e)
@@ -1087,30 +1162,28 @@ int prepare_kernels(fr_mesh* m) {
     hex_dispatch(m->order, [&](auto n) {
       constexpr int N = decltype(n)::value;
       constexpr int E = hex_epb<N>();
-      cudaFuncSetAttribute(k_hex_vol<T, TR, N, E, false>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           int(hex_vol_smem<T, TR, N>()));
-      cudaFuncSetAttribute(k_hex_vol<T, TR, N, E, true>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           int(hex_vol_smem<T, TR, N>()));
-      cudaFuncSetAttribute(k_hex_vol<T, TR, N, E, false, true>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           int(hex_vol_smem<T, TR, N>()));
-      cudaFuncSetAttribute(k_hex_vol<T, TR, N, E, true, true>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           int(hex_vol_smem<T, TR, N>()));
-      cudaFuncSetAttribute(k_hex_grad<T, TR, N, E, sizeof(T) == 4>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           int(hex_grad_smem<T, N>()));
-      cudaFuncSetAttribute(k_hex_grad_v<T, TR, N, E>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           int(hexv_grad_smem<T, N>()));
-      cudaFuncSetAttribute(k_hex_vol_v<T, TR, N, E, false>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           int(hexv_vol_smem<T, TR, N>()));
-      cudaFuncSetAttribute(k_hex_vol_v<T, TR, N, E, true>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           int(hexv_vol_smem<T, TR, N>()));
+      if constexpr (use_hexfx<T, N>()) {
+        const int sg = E * hexfx_bytes_per_elem<N>(true), sv = E * hexfx_bytes_per_elem<N>(false);
+        for (auto fn : {k_hexfx_grad<N, E, false>, k_hexfx_grad<N, E, true>})
+          cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, sg);
+        for (auto fn : {k_hexfx_vol<N, E, false>, k_hexfx_vol<N, E, true>,
+                        k_hexfx_vol<N, E, false, true>})
+          cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, sv);
+      } else {
+        const int sv = int(hex_vol_smem<T, TR, N>());
+        for (auto fn : {k_hex_vol<T, TR, N, E, false>, k_hex_vol<T, TR, N, E, true>,
+                        k_hex_vol<T, TR, N, E, false, true>, k_hex_vol<T, TR, N, E, true, true>})
+          cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, sv);
+        cudaFuncSetAttribute(k_hex_grad<T, TR, N, E, sizeof(T) == 4>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             int(hex_grad_smem<T, N>()));
+        cudaFuncSetAttribute(k_hex_grad_v<T, TR, N, E>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             int(hexv_grad_smem<T, N>()));
+        const int svv = int(hexv_vol_smem<T, TR, N>());
+        for (auto fn : {k_hex_vol_v<T, TR, N, E, false>, k_hex_vol_v<T, TR, N, E, true>})
+          cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, svv);
+      }
     });
   }
   CK(cudaGetLastError());
@@ -1220,6 +1293,9 @@ inline DevType sub_view(const fr_mesh* m, const DevType& D, long long e0, long l
   V.R = sh(D.R, 5 * nu * w);
   V.smat = sh(D.smat, 9 * nu * w);
   V.rcpdjac = sh(D.rcpdjac, nu * w);
+  V.fxs = static_cast<FxCoef*>(sh(D.fxs, 9 * nu * sizeof(FxCoef)));
+  V.fxj = static_cast<FxCoef*>(sh(D.fxj, 9 * nu * sizeof(FxCoef)));
+  V.fxe = static_cast<int*>(sh(D.fxe, 4 * sizeof(int)));
   V.grad = sh(D.grad, 15 * nu * w);
   V.fnv = sh(D.fnv, 3 * nf * w);
   V.fbc = static_cast<int8_t*>(sh(D.fbc, nf));
@@ -1333,11 +1409,22 @@ void launch_stage(fr_mesh* m, cudaStream_t s, int mode, int stage,
           constexpr int N = decltype(n)::value;
           constexpr int E = hex_epb<N>();
           const int eb = D.tile_grad > 0 ? D.tile_grad : E;
-          k_hex_grad<T, TR, N, E, sizeof(T) == 4>
-              <<<nblk(D.ne, eb), eb * N * N * N, hex_grad_smem<T, N>() / E * eb, s>>>(
-                  D.ne, from_x ? nullptr : (const T*)D.Y, (const TR*)D.X, du,
-                  (const T*)D.smat, (const T*)D.rcpdjac, hexops<T>(D),
-                  (T*)D.grad, va, bc, ph);
+          if constexpr (use_hexfx<T, N>()) {
+            const unsigned grid = nblk(D.ne, eb), tpb = eb * FxGeom<N>::TPE;
+            const size_t sm = size_t(eb) * hexfx_bytes_per_elem<N>(true);
+            const T* uin = from_x ? (const T*)D.X : (const T*)D.Y;
+            if (m->aa_qdeg > 0)
+              k_hexfx_grad<N, E, true><<<grid, tpb, sm, s>>>(D.ne, uin, du, D.fxj, D.fxe, D.hxfx,
+                                                             ph, (T*)D.grad, va.q);
+            else
+              k_hexfx_grad<N, E, false><<<grid, tpb, sm, s>>>(D.ne, uin, du, D.fxj, D.fxe, D.hxfx,
+                                                              ph, (T*)D.grad, va.q);
+          } else
+            k_hex_grad<T, TR, N, E, sizeof(T) == 4>
+                <<<nblk(D.ne, eb), eb * N * N * N, hex_grad_smem<T, N>() / E * eb, s>>>(
+                    D.ne, from_x ? nullptr : (const T*)D.Y, (const TR*)D.X, du,
+                    (const T*)D.smat, (const T*)D.rcpdjac, hexops<T>(D),
+                    (T*)D.grad, va, bc, ph);
         });
       } else if (use_tc_grad(m, D)) {
         launch_grad_tc<T, TR>(m, D, s, from_x, du, va, bc, ph);
@@ -1423,35 +1510,52 @@ void launch_stage(fr_mesh* m, cudaStream_t s, int mode, int stage,
         constexpr int N = decltype(n)::value;
         constexpr int E = hex_epb<N>();
         const int eb = D.tile_vol > 0 ? D.tile_vol : E;
-        const size_t sm = hex_vol_smem<T, TR, N>() / E * eb;
-        const T* uin = from_x ? nullptr : (const T*)D.Y;
-        if (sizeof(T) == 4 && D.verts && m->active == FR_VARIANT_SUMFACT_VERTEX) {
-          const size_t smv = hexv_vol_smem<T, TR, N>() / E * eb;
-          const T* dup = (const T*)m->du + D.off_f;
-          if (ns)
-            k_hex_vol_v<T, TR, N, E, true><<<nblk(D.ne, eb), eb * N * N * N, smv, s>>>(
-                D.ne, uin, dup, fc, (const T*)D.verts, hexops<T>(D), ph, sa);
+        if constexpr (use_hexfx<T, N>()) {
+          const size_t sm = size_t(eb) * hexfx_bytes_per_elem<N>(false);
+          const unsigned grid = nblk(D.ne, eb), tpb = eb * FxGeom<N>::TPE;
+          const T* uin = from_x ? (const T*)D.X : (const T*)D.Y;
+          if (aa)
+            k_hexfx_vol<N, E, false, true><<<grid, tpb, sm, s>>>(
+                D.ne, uin, nullptr, fc, nullptr, nullptr, (const T*)D.rcpdjac, D.hxfx, ph, sa,
+                (const T*)D.tf);
+          else if (ns)
+            k_hexfx_vol<N, E, true><<<grid, tpb, sm, s>>>(
+                D.ne, uin, (const T*)D.grad, fc, D.fxs, D.fxe, (const T*)D.rcpdjac,
+                D.hxfx, ph, sa);
           else
-            k_hex_vol_v<T, TR, N, E, false><<<nblk(D.ne, eb), eb * N * N * N, smv, s>>>(
-                D.ne, uin, nullptr, fc, (const T*)D.verts, hexops<T>(D), ph, sa);
-          return;
+            k_hexfx_vol<N, E, false><<<grid, tpb, sm, s>>>(
+                D.ne, uin, nullptr, fc, D.fxs, D.fxe, (const T*)D.rcpdjac, D.hxfx, ph, sa);
+        } else {
+          const size_t sm = hex_vol_smem<T, TR, N>() / E * eb;
+          const T* uin = from_x ? nullptr : (const T*)D.Y;
+          if (sizeof(T) == 4 && D.verts && m->active == FR_VARIANT_SUMFACT_VERTEX) {
+            const size_t smv = hexv_vol_smem<T, TR, N>() / E * eb;
+            const T* dup = (const T*)m->du + D.off_f;
+            if (ns)
+              k_hex_vol_v<T, TR, N, E, true><<<nblk(D.ne, eb), eb * N * N * N, smv, s>>>(
+                  D.ne, uin, dup, fc, (const T*)D.verts, hexops<T>(D), ph, sa);
+            else
+              k_hex_vol_v<T, TR, N, E, false><<<nblk(D.ne, eb), eb * N * N * N, smv, s>>>(
+                  D.ne, uin, nullptr, fc, (const T*)D.verts, hexops<T>(D), ph, sa);
+            return;
+          }
+          if (aa && ns)
+            k_hex_vol<T, TR, N, E, true, true><<<nblk(D.ne, eb), eb * N * N * N, sm, s>>>(
+                D.ne, uin, nullptr, fc, nullptr, (const T*)D.rcpdjac, hexops<T>(D),
+                ph, sa, (const T*)D.tf);
+          else if (aa)
+            k_hex_vol<T, TR, N, E, false, true><<<nblk(D.ne, eb), eb * N * N * N, sm, s>>>(
+                D.ne, uin, nullptr, fc, nullptr, (const T*)D.rcpdjac, hexops<T>(D),
+                ph, sa, (const T*)D.tf);
+          else if (ns)
+            k_hex_vol<T, TR, N, E, true><<<nblk(D.ne, eb), eb * N * N * N, sm, s>>>(
+                D.ne, uin, (const T*)D.grad, fc, (const T*)D.smat,
+                (const T*)D.rcpdjac, hexops<T>(D), ph, sa);
+          else
+            k_hex_vol<T, TR, N, E, false><<<nblk(D.ne, eb), eb * N * N * N, sm, s>>>(
+                D.ne, uin, nullptr, fc, (const T*)D.smat, (const T*)D.rcpdjac,
+                hexops<T>(D), ph, sa);
         }
-        if (aa && ns)
-          k_hex_vol<T, TR, N, E, true, true><<<nblk(D.ne, eb), eb * N * N * N, sm, s>>>(
-              D.ne, uin, nullptr, fc, nullptr, (const T*)D.rcpdjac, hexops<T>(D),
-              ph, sa, (const T*)D.tf);
-        else if (aa)
-          k_hex_vol<T, TR, N, E, false, true><<<nblk(D.ne, eb), eb * N * N * N, sm, s>>>(
-              D.ne, uin, nullptr, fc, nullptr, (const T*)D.rcpdjac, hexops<T>(D),
-              ph, sa, (const T*)D.tf);
-        else if (ns)
-          k_hex_vol<T, TR, N, E, true><<<nblk(D.ne, eb), eb * N * N * N, sm, s>>>(
-              D.ne, uin, (const T*)D.grad, fc, (const T*)D.smat,
-              (const T*)D.rcpdjac, hexops<T>(D), ph, sa);
-        else
-          k_hex_vol<T, TR, N, E, false><<<nblk(D.ne, eb), eb * N * N * N, sm, s>>>(
-              D.ne, uin, nullptr, fc, (const T*)D.smat, (const T*)D.rcpdjac,
-              hexops<T>(D), ph, sa);
       });
     } else if (use_tc_vol(m, D)) {
       HexStage<T, TR> sa{mode, stage, (TR*)D.X, (TR*)D.A, (T*)D.Y, (T*)D.R,

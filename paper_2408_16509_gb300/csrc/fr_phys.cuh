@@ -114,6 +114,57 @@ __device__ __forceinline__ void viscous_flux_acc(const T u[5], const T g[3][5],
   }
 }
 
+// Viscous flux at a point: stress (xx, yy, zz, xy, xz, yz) in tq[0..5] and
+// energy flux v.tau + kappa grad e in tq[6..8].  The velocity gradient is
+// left undivided by rho (d[j][i] = g_j(m_i) - v_i g_j(rho)): one factor
+// mu / rho on the six stresses.
+template <typename T>
+__device__ __forceinline__ void viscous_point(const T u[5], const T (&g)[3][5],
+                                              const Phys<T>& ph, T tq[9]) {
+  const T ri = T(1) / u[0];
+  const T v[3] = {u[1] * ri, u[2] * ri, u[3] * ri};
+  const T er = u[4] * ri, mr = ph.mu * ri, kr = ph.kappa * ri;
+  T d[3][3];
+#pragma unroll
+  for (int j = 0; j < 3; ++j)
+#pragma unroll
+    for (int i = 0; i < 3; ++i) d[j][i] = g[j][1 + i] - v[i] * g[j][0];
+  const T m2 = T(2) * mr;
+  const T dv = (T(2.0 / 3.0) * mr) * (d[0][0] + d[1][1] + d[2][2]);
+#pragma unroll
+  for (int j = 0; j < 3; ++j) tq[j] = m2 * d[j][j] - dv;
+  tq[3] = mr * (d[0][1] + d[1][0]);
+  tq[4] = mr * (d[0][2] + d[2][0]);
+  tq[5] = mr * (d[1][2] + d[2][1]);
+  const T t[3][3] = {{tq[0], tq[3], tq[4]}, {tq[3], tq[1], tq[5]}, {tq[4], tq[5], tq[2]}};
+#pragma unroll
+  for (int j = 0; j < 3; ++j)
+    tq[6 + j] = kr * ((g[j][4] - er * g[j][0]) -
+                      (v[0] * d[j][0] + v[1] * d[j][1] + v[2] * d[j][2])) +
+                (v[0] * t[j][0] + v[1] * t[j][1] + v[2] * t[j][2]);
+}
+
+// Total flux at a point, the 12 distinct values of F[j][k]: mass (the
+// momentum) f[0..2], momentum f[3..8] (xx, yy, zz, xy, xz, yz), energy
+// f[9..11]; tq: viscous_point's values (NS).
+template <typename T, bool NS>
+__device__ __forceinline__ void flux_point(const T u[5], const T tq[9], const Phys<T>& ph,
+                                           T f[12]) {
+  const T ri = T(1) / u[0];
+  const T v[3] = {u[1] * ri, u[2] * ri, u[3] * ri};
+  const T p = ph.gm1 * (u[4] - T(0.5) * (u[1] * v[0] + u[2] * v[1] + u[3] * v[2]));
+  const T h = u[4] + p;
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    f[j] = u[1 + j];
+    f[3 + j] = u[1 + j] * v[j] + (NS ? p - tq[j] : p);
+    f[9 + j] = NS ? h * v[j] - tq[6 + j] : h * v[j];
+  }
+  f[6] = NS ? u[1] * v[1] - tq[3] : u[1] * v[1];
+  f[7] = NS ? u[1] * v[2] - tq[4] : u[1] * v[2];
+  f[8] = NS ? u[2] * v[2] - tq[5] : u[2] * v[2];
+}
+
 // normal viscous flux n.Fv accumulated into f[k] with sign sgn, formed
 // directly: (tau n)_i = mu (sum_j (dv_i/dx_j + dv_j/dx_i) n_j - 2/3 div v n_i),
 // energy v.(tau n) + kappa n.grad e (the full tensor is never built).
