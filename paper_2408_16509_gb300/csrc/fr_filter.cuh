@@ -232,11 +232,9 @@ __global__ void k_entropy_min(long long ne, const T* __restrict__ uin,
     if (i < NU + 2 * NF) {
       const int32_t c = partner[e * NF + (i - NU - NF)];
       if (c < 0) return false;
-      int t2, f2;
-      long long e2;
-      decode_fp(c, tt, &t2, &e2, &f2);
+      const FluxPt p(c, tt);
 #pragma unroll
-      for (int k = 0; k < 5; ++k) v[k] = V(uf_all[fp_index(tt, t2, e2, f2, 5, k)]);
+      for (int k = 0; k < 5; ++k) v[k] = V(uf_all[p.p5 + (long long)k * p.nf]);
       return true;
     }
     return false;

@@ -99,22 +99,26 @@ static __constant__ float c_rk45_ef[5] = {
     float(2114624349019.0 / 3568978502595.0 - 606302364029.0 / 971179775848.0),
     float(5198255086312.0 / 14908931495163.0 - 1097981568119.0 / 3980877426909.0)};
 
-__device__ __forceinline__ void decode_fp(int32_t code, const TypeTab& tt,
-                                          int* t, long long* e, int* f) {
-  *t = code >> 29;
-  long long local = code & ((1 << 29) - 1);
-  int nf = tt.nf[*t];
-  *e = local / (5 * nf);
-  *f = int(local - *e * 5 * nf);
-}
-
-// index of variable v, point f, element e in a [ne][nv][nf] region of type t
-__device__ __forceinline__ long long fp_index(const TypeTab& tt, int t,
-                                              long long e, int f, int nv,
-                                              int v) {
-  long long base = tt.off_f[t] / 5 * nv;  // region scales with the var count
-  return base + (e * nv + v) * tt.nf[t] + f;
-}
+// A flux-point code (type in bits 29-30, e 5 nf + f below) as a position in
+// the flux-point buffers.  In a [ne][5][nf] region variable k of the point
+// is at p5 + k nf without any division; in a [ne][15][nf] region component c
+// is at p15() + c nf, which needs f = code mod nf (a 32-bit remainder).
+struct FluxPt {
+  long long p5;
+  int nf;
+  unsigned local;
+  __device__ __forceinline__ FluxPt(int32_t code, const TypeTab& tt) {
+    const int t = code >> 29;
+    local = unsigned(code) & ((1u << 29) - 1);
+    nf = tt.nf[t];
+    p5 = tt.off_f[t] + local;
+  }
+  __device__ __forceinline__ long long p15() const {
+    return 3 * p5 - 2 * (long long)(local % unsigned(nf));
+  }
+  // position of component 0 in a [ne][nv][nf] region, nv = 5 or 15
+  __device__ __forceinline__ long long at(int nv) const { return nv == 5 ? p5 : p15(); }
+};
 
 // RK epilogue for one point: R[5] -> registers; returns the next stage value
 template <typename T>
@@ -241,15 +245,12 @@ __global__ void k_face_flux(int np, const int32_t* __restrict__ pl,
                             T* __restrict__ fc, TypeTab tt, Phys<T> ph) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= np) return;
-  int tl, tr, fl, frr;
-  long long el, er;
-  decode_fp(pl[i], tt, &tl, &el, &fl);
-  decode_fp(pr[i], tt, &tr, &er, &frr);
+  const FluxPt L(pl[i], tt), R(pr[i], tt);
   T ul[5], ur[5], n[3];
 #pragma unroll
   for (int k = 0; k < 5; ++k) {
-    ul[k] = uf[fp_index(tt, tl, el, fl, 5, k)];
-    ur[k] = uf[fp_index(tt, tr, er, frr, 5, k)];
+    ul[k] = uf[L.p5 + (long long)k * L.nf];
+    ur[k] = uf[R.p5 + (long long)k * R.nf];
   }
   n[0] = pn[4 * i];
   n[1] = pn[4 * i + 1];
@@ -259,12 +260,14 @@ __global__ void k_face_flux(int np, const int32_t* __restrict__ pl,
   rusanov(ul, ur, n, ph, F);
   if (NS) {
     T gl[3][5], gr[3][5];
+    const T* pgl = gf + L.p15();
+    const T* pgr = gf + R.p15();
 #pragma unroll
     for (int j = 0; j < 3; ++j)
 #pragma unroll
       for (int k = 0; k < 5; ++k) {
-        gl[j][k] = gf[fp_index(tt, tl, el, fl, 15, j * 5 + k)];
-        gr[j][k] = gf[fp_index(tt, tr, er, frr, 15, j * 5 + k)];
+        gl[j][k] = pgl[(j * 5 + k) * L.nf];
+        gr[j][k] = pgr[(j * 5 + k) * R.nf];
       }
     viscous_normal_acc(ul, gl, n, ph, -(T(0.5) + ph.beta), F);
     viscous_normal_acc(ur, gr, n, ph, -(T(0.5) - ph.beta), F);
@@ -273,8 +276,8 @@ __global__ void k_face_flux(int np, const int32_t* __restrict__ pl,
   }
 #pragma unroll
   for (int k = 0; k < 5; ++k) {
-    fc[fp_index(tt, tl, el, fl, 5, k)] = ml * F[k];
-    fc[fp_index(tt, tr, er, frr, 5, k)] = -mr * F[k];
+    fc[L.p5 + (long long)k * L.nf] = ml * F[k];
+    fc[R.p5 + (long long)k * R.nf] = -mr * F[k];
   }
 }
 
@@ -318,12 +321,10 @@ __global__ void k_bnd_flux(int nb, const int32_t* __restrict__ bidx,
                            const T* __restrict__ xg = nullptr) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nb) return;
-  int t, f;
-  long long e;
-  decode_fp(bidx[i], tt, &t, &e, &f);
+  const FluxPt p(bidx[i], tt);
   T ul[5], ur[5], n[3] = {bn[4 * i], bn[4 * i + 1], bn[4 * i + 2]};
 #pragma unroll
-  for (int k = 0; k < 5; ++k) ul[k] = uf[fp_index(tt, t, e, f, 5, k)];
+  for (int k = 0; k < 5; ++k) ul[k] = uf[p.p5 + (long long)k * p.nf];
   const int b = bbc[i];
   ghost_state_x(bc, b, i, xu, ul, ur);
   T F[5];
@@ -331,11 +332,12 @@ __global__ void k_bnd_flux(int nb, const int32_t* __restrict__ bidx,
   if (NS) {
     T g[3][5], gr[3][5];
     const bool x = bc.kind[b] == 2;
+    const T* pg = gf + p.p15();
 #pragma unroll
     for (int j = 0; j < 3; ++j)
 #pragma unroll
       for (int k = 0; k < 5; ++k) {
-        g[j][k] = gf[fp_index(tt, t, e, f, 15, j * 5 + k)];
+        g[j][k] = pg[(j * 5 + k) * p.nf];
         gr[j][k] = x ? xg[15 * i + j * 5 + k] : g[j][k];
       }
     const T vb = x ? T(0) : ph.beta;  // exchange points: BR1 weights
@@ -346,7 +348,7 @@ __global__ void k_bnd_flux(int nb, const int32_t* __restrict__ bidx,
   }
   T m = bn[4 * i + 3];
 #pragma unroll
-  for (int k = 0; k < 5; ++k) fc[fp_index(tt, t, e, f, 5, k)] = m * F[k];
+  for (int k = 0; k < 5; ++k) fc[p.p5 + (long long)k * p.nf] = m * F[k];
 }
 
 // NS: common solution u^C = (u- + u+)/2; stores u^C - u_f on both sides.
@@ -358,14 +360,10 @@ __global__ void k_face_ucommon(int np, const int32_t* __restrict__ pl,
                                TypeTab tt, T beta = T(0)) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= np) return;
-  int tl, tr, fl, frr;
-  long long el, er;
-  decode_fp(pl[i], tt, &tl, &el, &fl);
-  decode_fp(pr[i], tt, &tr, &er, &frr);
+  const FluxPt L(pl[i], tt), R(pr[i], tt);
 #pragma unroll
   for (int k = 0; k < 5; ++k) {
-    long long il = fp_index(tt, tl, el, fl, 5, k);
-    long long ir = fp_index(tt, tr, er, frr, 5, k);
+    const long long il = L.p5 + (long long)k * L.nf, ir = R.p5 + (long long)k * R.nf;
     T a = uf[il], b = uf[ir];
     du[il] = (T(0.5) + beta) * (b - a);
     du[ir] = -(T(0.5) - beta) * (b - a);
@@ -380,18 +378,16 @@ __global__ void k_bnd_ucommon(int nb, const int32_t* __restrict__ bidx,
                               const T* __restrict__ xu = nullptr, T ph_beta = T(0)) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nb) return;
-  int t, f;
-  long long e;
-  decode_fp(bidx[i], tt, &t, &e, &f);
+  const FluxPt p(bidx[i], tt);
   T ul[5], ur[5];
 #pragma unroll
-  for (int k = 0; k < 5; ++k) ul[k] = uf[fp_index(tt, t, e, f, 5, k)];
+  for (int k = 0; k < 5; ++k) ul[k] = uf[p.p5 + (long long)k * p.nf];
   const int b = bbc[i];
   ghost_state_x(bc, b, i, xu, ul, ur);
   const T w = bc.kind[b] == 2 ? T(0.5) : T(0.5) + ph_beta;
 #pragma unroll
   for (int k = 0; k < 5; ++k)
-    du[fp_index(tt, t, e, f, 5, k)] = w * (ur[k] - ul[k]);
+    du[p.p5 + (long long)k * p.nf] = w * (ur[k] - ul[k]);
 }
 
 // ---------------------------------------------------------------------------
@@ -504,15 +500,11 @@ __global__ void k_face_flux_ns(int np, const int32_t* __restrict__ pl,
                                TypeTab tt, Phys<T> ph) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= np) return;
-  int tl, tr, fl, frr;
-  long long el, er;
-  decode_fp(pl[i], tt, &tl, &el, &fl);
-  decode_fp(pr[i], tt, &tr, &er, &frr);
+  const FluxPt L(pl[i], tt), R(pr[i], tt);
   T ul[5], ur[5], ql[5], qr[5];
 #pragma unroll
   for (int k = 0; k < 5; ++k) {
-    long long il = fp_index(tt, tl, el, fl, 5, k);
-    long long ir = fp_index(tt, tr, er, frr, 5, k);
+    const long long il = L.p5 + (long long)k * L.nf, ir = R.p5 + (long long)k * R.nf;
     ul[k] = uf[il];
     ur[k] = uf[ir];
     ql[k] = q[il];
@@ -527,8 +519,8 @@ __global__ void k_face_flux_ns(int np, const int32_t* __restrict__ pl,
 #pragma unroll
   for (int k = 0; k < 5; ++k) {
     const T G = F[k] + ph.tau * (ul[k] - ur[k]);
-    fc[fp_index(tt, tl, el, fl, 5, k)] = ml * G - (wl * ql[k] - wr * rl * qr[k]);
-    fc[fp_index(tt, tr, er, frr, 5, k)] = -mr * G + (wl * rr * ql[k] - wr * qr[k]);
+    fc[L.p5 + (long long)k * L.nf] = ml * G - (wl * ql[k] - wr * rl * qr[k]);
+    fc[R.p5 + (long long)k * R.nf] = -mr * G + (wl * rr * ql[k] - wr * qr[k]);
   }
 }
 
@@ -547,12 +539,10 @@ __global__ void k_bnd_flux_ns(int nb, const int32_t* __restrict__ bidx,
                               const T* __restrict__ xm = nullptr) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nb) return;
-  int t, f;
-  long long e;
-  decode_fp(bidx[i], tt, &t, &e, &f);
+  const FluxPt p(bidx[i], tt);
   T ul[5], ur[5], n[3] = {bn[4 * i], bn[4 * i + 1], bn[4 * i + 2]};
 #pragma unroll
-  for (int k = 0; k < 5; ++k) ul[k] = uf[fp_index(tt, t, e, f, 5, k)];
+  for (int k = 0; k < 5; ++k) ul[k] = uf[p.p5 + (long long)k * p.nf];
   const int b = bbc[i];
   ghost_state_x(bc, b, i, xu, ul, ur);
   T F[5];
@@ -562,14 +552,14 @@ __global__ void k_bnd_flux_ns(int nb, const int32_t* __restrict__ bidx,
     const T rl = m / xm[i];
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
-      long long ix = fp_index(tt, t, e, f, 5, k);
+      const long long ix = p.p5 + (long long)k * p.nf;
       fc[ix] = m * (F[k] + ph.tau * (ul[k] - ur[k])) - T(0.5) * (q[ix] - rl * xq[5 * i + k]);
     }
     return;
   }
 #pragma unroll
   for (int k = 0; k < 5; ++k) {
-    long long ix = fp_index(tt, t, e, f, 5, k);
+    const long long ix = p.p5 + (long long)k * p.nf;
     fc[ix] = m * (F[k] + ph.tau * (ul[k] - ur[k])) - q[ix];
   }
 }
@@ -586,11 +576,10 @@ __global__ void k_exchange_push(int n, const int32_t* __restrict__ code,
                                 T* const* __restrict__ dst, TypeTab tt) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  int t, f;
-  long long e;
-  decode_fp(code[i], tt, &t, &e, &f);
+  const FluxPt p(code[i], tt);
+  const T* v = src + p.at(nv);
   T* d = dst[to[i]] + (long long)slot[i] * nv;
-  for (int c = 0; c < nv; ++c) d[c] = src[fp_index(tt, t, e, f, nv, c)];
+  for (int c = 0; c < nv; ++c) d[c] = v[(long long)c * p.nf];
 }
 
 // Exchange with other processes: gather the traces (nv values per point) at
@@ -603,10 +592,9 @@ __global__ void k_exchange_gather(int n, const int32_t* __restrict__ list,
                                   T* __restrict__ dst, TypeTab tt) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  int t, f;
-  long long e;
-  decode_fp(bidx[list[i]], tt, &t, &e, &f);
-  for (int c = 0; c < nv; ++c) dst[(long long)i * nv + c] = src[fp_index(tt, t, e, f, nv, c)];
+  const FluxPt p(bidx[list[i]], tt);
+  const T* v = src + p.at(nv);
+  for (int c = 0; c < nv; ++c) dst[(long long)i * nv + c] = v[(long long)c * p.nf];
 }
 
 template <typename T>

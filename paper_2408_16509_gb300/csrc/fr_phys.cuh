@@ -31,36 +31,29 @@ __device__ __forceinline__ double fr_sqrt<double>(double x) { return sqrt(x); }
 template <>
 __device__ __forceinline__ float fr_sqrt<float>(float x) { return sqrtf(x); }
 
-// normal inviscid flux n.F(u), pressure and normal velocity
-template <typename T>
-__device__ __forceinline__ void normal_flux(const T u[5], const T n[3],
-                                            const Phys<T>& ph, T fn[5], T* c,
-                                            T* vn) {
-  T ri = T(1) / u[0];
-  T vx = u[1] * ri, vy = u[2] * ri, vz = u[3] * ri;
-  T p = ph.gm1 * (u[4] - T(0.5) * (u[1] * vx + u[2] * vy + u[3] * vz));
-  T v = vx * n[0] + vy * n[1] + vz * n[2];
-  fn[0] = u[0] * v;
-  fn[1] = u[1] * v + p * n[0];
-  fn[2] = u[2] * v + p * n[1];
-  fn[3] = u[3] * v + p * n[2];
-  fn[4] = (u[4] + p) * v;
-  *c = fr_sqrt<T>(ph.gamma * p * ri);
-  *vn = v;
-}
-
+// Rusanov flux along n.  Both sides' inviscid fluxes are added before the
+// halving and the velocity components are never formed (n.m and m.m of the
+// momentum m serve the flux, the pressure and the wave speed): 89 FP64
+// instructions a pair with the two reciprocals and roots, 100 with one flux
+// per side.
 template <typename T>
 __device__ __forceinline__ void rusanov(const T ul[5], const T ur[5],
                                         const T n[3], const Phys<T>& ph,
                                         T F[5]) {
-  T fl[5], fr[5], cl, cr, vl, vr;
-  normal_flux(ul, n, ph, fl, &cl, &vl);
-  normal_flux(ur, n, ph, fr, &cr, &vr);
-  T a = fabs(vl) + cl, b = fabs(vr) + cr;
-  T lam = a > b ? a : b;
+  const T il = T(1) / ul[0], ir = T(1) / ur[0];
+  const T ml = ul[1] * n[0] + ul[2] * n[1] + ul[3] * n[2];
+  const T mr = ur[1] * n[0] + ur[2] * n[1] + ur[3] * n[2];
+  const T vl = ml * il, vr = mr * ir;
+  const T pl = ph.gm1 * (ul[4] - (T(0.5) * il) * (ul[1] * ul[1] + ul[2] * ul[2] + ul[3] * ul[3]));
+  const T pr = ph.gm1 * (ur[4] - (T(0.5) * ir) * (ur[1] * ur[1] + ur[2] * ur[2] + ur[3] * ur[3]));
+  const T a = fabs(vl) + fr_sqrt<T>(ph.gamma * pl * il);
+  const T b = fabs(vr) + fr_sqrt<T>(ph.gamma * pr * ir);
+  const T hl = T(0.5) * (a > b ? a : b), ps = pl + pr;
+  F[0] = T(0.5) * (ml + mr) + hl * (ul[0] - ur[0]);
 #pragma unroll
-  for (int k = 0; k < 5; ++k)
-    F[k] = T(0.5) * (fl[k] + fr[k]) - T(0.5) * lam * (ur[k] - ul[k]);
+  for (int k = 0; k < 3; ++k)
+    F[1 + k] = T(0.5) * (ul[1 + k] * vl + ur[1 + k] * vr + ps * n[k]) + hl * (ul[1 + k] - ur[1 + k]);
+  F[4] = T(0.5) * ((ul[4] + pl) * vl + (ur[4] + pr) * vr) + hl * (ul[4] - ur[4]);
 }
 
 // inviscid flux F[j][k] in direction j of variable k
@@ -165,41 +158,72 @@ __device__ __forceinline__ void flux_point(const T u[5], const T tq[9], const Ph
   f[8] = NS ? u[2] * v[2] - tq[5] : u[2] * v[2];
 }
 
-// normal viscous flux n.Fv accumulated into f[k] with sign sgn, formed
-// directly: (tau n)_i = mu (sum_j (dv_i/dx_j + dv_j/dx_i) n_j - 2/3 div v n_i),
-// energy v.(tau n) + kappa n.grad e (the full tensor is never built).
+// Normal viscous flux n.Fv accumulated into f[k] with weight wt.
+// FP64: formed from the gradients along n (gn_k = n.grad u_k) and their
+// transpose: with x_i = gn_i - v_i gn_0 + sum_j n_j (g_i(m_j) - v_j g_i(rho))
+// - 2/3 n_i (div m - v.grad rho), (tau n)_i = (mu / rho) x_i, energy
+// (mu / rho) v.x + (kappa / rho) rho n.grad e.  The velocity gradient is
+// never built: 59 instructions a side against 75 (interface kernel, FP64-pipe
+// bound, 24^3 p = 4: 485 -> 447 us with the Rusanov form above).
+// FP32: (tau n)_i = mu (sum_j (dv_i/dx_j + dv_j/dx_i) n_j - 2/3 div v n_i) from
+// the velocity gradient; the form above made the prism and tetrahedron
+// gradient kernels 1 % slower.
 template <typename T>
 __device__ __forceinline__ void viscous_normal_acc(const T u[5],
                                                    const T g[3][5],
                                                    const T n[3],
-                                                   const Phys<T>& ph, T sgn,
+                                                   const Phys<T>& ph, T wt,
                                                    T f[5]) {
-  const T ri = T(1) / u[0];
-  const T v[3] = {u[1] * ri, u[2] * ri, u[3] * ri};
-  const T er = u[4] * ri;
-  T gv[3][3];  // gv[j][i] = d v_i / d x_j
-  T gen = T(0);  // n . grad e
+  if constexpr (sizeof(T) == 8) {
+    const T ri = T(1) / u[0];
+    const T v[3] = {u[1] * ri, u[2] * ri, u[3] * ri};
+    const T er = u[4] * ri, mr = wt * (ph.mu * ri), kr = wt * (ph.kappa * ri);
+    T gn[5];
 #pragma unroll
-  for (int j = 0; j < 3; ++j) {
+    for (int k = 0; k < 5; ++k) gn[k] = n[0] * g[0][k] + n[1] * g[1][k] + n[2] * g[2][k];
+    const T vn = v[0] * n[0] + v[1] * n[1] + v[2] * n[2];
+    const T div = (g[0][1] + g[1][2] + g[2][3]) -
+                  (v[0] * g[0][0] + v[1] * g[1][0] + v[2] * g[2][0]);
+    const T d23 = T(2.0 / 3.0) * div;
+    T vx = T(0), vt = T(0);
 #pragma unroll
-    for (int i = 0; i < 3; ++i) gv[j][i] = (g[j][1 + i] - v[i] * g[j][0]) * ri;
-    const T ge = (g[j][4] - er * g[j][0]) * ri -
-                 (v[0] * gv[j][0] + v[1] * gv[j][1] + v[2] * gv[j][2]);
-    gen += n[j] * ge;
+    for (int i = 0; i < 3; ++i) {
+      const T t = gn[1 + i] - v[i] * gn[0];
+      const T s = n[0] * g[i][1] + n[1] * g[i][2] + n[2] * g[i][3] - vn * g[i][0];
+      const T x = t + (s - d23 * n[i]);
+      f[1 + i] += mr * x;
+      vx += v[i] * x;
+      vt += v[i] * t;
+    }
+    f[4] += mr * vx + kr * ((gn[4] - er * gn[0]) - vt);
+  } else {
+    const T ri = T(1) / u[0];
+    const T v[3] = {u[1] * ri, u[2] * ri, u[3] * ri};
+    const T er = u[4] * ri;
+    T gv[3][3];  // gv[j][i] = d v_i / d x_j
+    T gen = T(0);  // n . grad e
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+#pragma unroll
+      for (int i = 0; i < 3; ++i) gv[j][i] = (g[j][1 + i] - v[i] * g[j][0]) * ri;
+      const T ge = (g[j][4] - er * g[j][0]) * ri -
+                   (v[0] * gv[j][0] + v[1] * gv[j][1] + v[2] * gv[j][2]);
+      gen += n[j] * ge;
+    }
+    const T div23 = T(2.0 / 3.0) * (gv[0][0] + gv[1][1] + gv[2][2]);
+    T tn[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      T s = -div23 * n[i];
+#pragma unroll
+      for (int j = 0; j < 3; ++j) s += (gv[j][i] + gv[i][j]) * n[j];
+      tn[i] = ph.mu * s;
+    }
+    f[1] += wt * tn[0];
+    f[2] += wt * tn[1];
+    f[3] += wt * tn[2];
+    f[4] += wt * (v[0] * tn[0] + v[1] * tn[1] + v[2] * tn[2] + ph.kappa * gen);
   }
-  const T div23 = T(2.0 / 3.0) * (gv[0][0] + gv[1][1] + gv[2][2]);
-  T tn[3];
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    T s = -div23 * n[i];
-#pragma unroll
-    for (int j = 0; j < 3; ++j) s += (gv[j][i] + gv[i][j]) * n[j];
-    tn[i] = ph.mu * s;
-  }
-  f[1] += sgn * tn[0];
-  f[2] += sgn * tn[1];
-  f[3] += sgn * tn[2];
-  f[4] += sgn * (v[0] * tn[0] + v[1] * tn[1] + v[2] * tn[2] + ph.kappa * gen);
 }
 
 }  // namespace frgb
