@@ -33,28 +33,7 @@ int setup_filter(fr_mesh* m) {
     if ((rc = dev_zeros(m, size_t(D.ne) * sizeof(int32_t), (void**)&D.flist))) return rc;
     if ((rc = dev_zeros(m, sizeof(int), (void**)&D.fcount))) return rc;
   }
-  // partner flux point of every element flux point (-1 on boundaries)
-  for (size_t t = 0; t < m->types.size(); ++t) {
-    DevType& D = m->types[t];
-    if (D.fpartner) continue;
-    std::vector<int32_t> part(size_t(D.ne) * D.nf, -1);
-    auto local = [&](int32_t code, int* tt, long long* e, int* f) {
-      *tt = code >> 29;
-      long long l = code & ((1 << 29) - 1);
-      int nfx = m->types[*tt].nf;
-      *e = l / (5 * nfx);
-      *f = int(l - *e * 5 * nfx);
-    };
-    for (size_t i = 0; i < m->conn.pl.size(); ++i) {
-      int ta, tb, fa, fb;
-      long long ea, eb;
-      local(m->conn.pl[i], &ta, &ea, &fa);
-      local(m->conn.pr[i], &tb, &eb, &fb);
-      if (ta == int(t)) part[size_t(ea) * D.nf + fa] = m->conn.pr[i];
-      if (tb == int(t)) part[size_t(eb) * D.nf + fb] = m->conn.pl[i];
-    }
-    if ((rc = dev_upload_i32(m, part, &D.fpartner))) return rc;
-  }
+  if ((rc = setup_partner(m))) return rc;
   if (!m->d_fstats) {
     if ((rc = dev_zeros(m, sizeof(FilterStats), (void**)&m->d_fstats))) return rc;
   }

@@ -156,8 +156,25 @@ __device__ __forceinline__ void hex_stage_apply(const HexStage<T, TR>& a,
     hex_stage_apply_mixed(a, i0, vstr, R, x, ac, s);
     return;
   }
-  const TR dt = TR(*a.dt);
+  // FP32 registers: dt and the coefficients rounded to FP32 without the FP64
+  // pipe (the same values)
   const int st = a.stage;
+  TR dt, b = TR(0), am = TR(0), ev = TR(0);
+  if constexpr (sizeof(TR) == 4) {
+    dt = narrow_f64(*a.dt);
+    if (a.mode == 2) {
+      b = c_rk45_bf[st];
+      am = st < 4 ? c_rk45_af[st] - b : 0.f;
+      ev = c_rk45_ef[st];
+    }
+  } else {
+    dt = *a.dt;
+    if (a.mode == 2) {
+      b = c_rk45_b[st];
+      am = st < 4 ? c_rk45_a[st] - b : 0.0;
+      ev = c_rk45_e[st];
+    }
+  }
   if (a.mode == 1) {
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
@@ -181,8 +198,6 @@ __device__ __forceinline__ void hex_stage_apply(const HexStage<T, TR>& a,
     }
     return;
   }
-  const TR b = TR(c_rk45_b[st]);
-  const TR am = st < 4 ? TR(c_rk45_a[st]) - b : TR(0);
 #pragma unroll
   for (int k = 0; k < 5; ++k) {
     const long long i = i0 + k * vstr;
@@ -190,8 +205,8 @@ __device__ __forceinline__ void hex_stage_apply(const HexStage<T, TR>& a,
     const TR xx = x[k] + b * dt * r;
     a.X[i] = xx;
     if (a.E) {  // error estimate dt sum_i (b_i - bhat_i) R_i
-      const TR ev = TR(c_rk45_e[st]) * dt * r;
-      a.E[i] = st == 0 ? ev : a.E[i] + ev;
+      const TR er = ev * dt * r;
+      a.E[i] = st == 0 ? er : a.E[i] + er;
     }
     if (st < 4) {
       const T y = T(xx + am * dt * r);
@@ -280,328 +295,6 @@ __device__ __forceinline__ void face_interp_pair(const T* src, int dir, int i, i
       const T v = src[k * NU + q];
       o0[k] += cm * v;
       o1[k] += cp * v;
-    }
-  }
-}
-
-// ---------------------------------------------------------------------------
-// NS gradients on hexahedra: corrected reference gradient, physical gradient
-// at solution points, and its value at the flux points.
-// QV: write the viscous normal flux q (5 per flux point, for the q-based
-// interface kernel) instead of the 15 gradient components at flux points.
-// Shared memory per element of k_hex_grad: u [5][NU], du [5][NF], physical
-// gradient [15][NU], and for the q form the traces [5][NF] and S^T n~
-// [3][NF] at the flux points (type T, 16-byte padded).
-template <typename T, int N, bool QV>
-__host__ __device__ constexpr int hex_grad_bytes_per_elem() {
-  return ((20 * N * N * N + (QV ? 78 : 30) * N * N) * int(sizeof(T)) + 15) / 16 * 16;
-}
-
-// The q form (FP32 values) is bounded to 64 registers at 250 threads so that
-// four CTAs fit on an SM (a few bytes spill; measured faster than three).
-template <typename T, typename TR, int N, int EPB, bool QV>
-__global__ void __launch_bounds__(EPB* N* N* N, (QV && EPB * N * N * N >= 250 ? 4 : 1))
-    k_hex_grad(long long ne, const T* __restrict__ uin, const TR* __restrict__ X,
-               const T* __restrict__ du, const T* __restrict__ smat,
-               const T* __restrict__ rcpdjac, HexOps<T> op,
-               T* __restrict__ grad, ViscArgs<T> va, BCTab<T> bc,
-               Phys<T> ph) {
-  constexpr int NU = N * N * N, NF = 6 * N * N;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int le = threadIdx.x / NU, z = threadIdx.x - le * NU;
-  const long long e = (long long)blockIdx.x * (blockDim.x / NU) + le;
-  T* us = reinterpret_cast<T*>(smem_raw + le * hex_grad_bytes_per_elem<T, N, QV>());
-  T* ds = us + 5 * NU;
-  T* gs = ds + 5 * NF;
-  T* ufs = gs + 15 * NU;  // [5][NF] traces (q form)
-  T* nvs = ufs + 5 * NF;  // [3][NF] S^T n~ (q form)
-  const int a = z % N, b = (z / N) % N, c = z / (N * N);
-  // the element's u, du (and the q form's inputs) arrive by cp.async while
-  // the metric terms load into registers
-  T S[3][3], rj = T(0);
-  if (e < ne) {
-    if (uin) {
-      async_copy(us, uin + e * 5 * NU, 5 * NU * int(sizeof(T)), z, NU);
-    } else {
-#pragma unroll
-      for (int k = 0; k < 5; ++k) us[k * NU + z] = T(X[(e * 5 + k) * NU + z]);
-    }
-    async_copy(ds, du + e * 5 * NF, 5 * NF * int(sizeof(T)), z, NU);
-    if (QV) {
-      async_copy(ufs, va.uf + e * 5 * NF, 5 * NF * int(sizeof(T)), z, NU);
-      async_copy(nvs, va.fnv + e * 3 * NF, 3 * NF * int(sizeof(T)), z, NU);
-    }
-#pragma unroll
-    for (int r = 0; r < 9; ++r) S[r / 3][r % 3] = smat[(e * 9 + r) * NU + z];
-    rj = rcpdjac[e * NU + z];
-  }
-  cp_async_wait_all();
-  __syncthreads();
-  if (e < ne) {
-    T gref[3][5];
-    const int N2 = N * N;
-    T da[N], db[N], dc[N];
-#pragma unroll
-    for (int m = 0; m < N; ++m) {
-      da[m] = op.d1[a][m];
-      db[m] = op.d1[b][m];
-      dc[m] = op.d1[c][m];
-    }
-    const T gla = op.gl[a], gra = op.gr[a], glb = op.gl[b], grb = op.gr[b],
-            glc = op.gl[c], grc = op.gr[c];
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-      T gx = T(0), gy = T(0), gz = T(0);
-#pragma unroll
-      for (int m = 0; m < N; ++m) {
-        gx += da[m] * us[k * NU + m + N * b + N2 * c];
-        gy += db[m] * us[k * NU + a + N * m + N2 * c];
-        gz += dc[m] * us[k * NU + a + N * b + N2 * m];
-      }
-      // correction: the face normal n~ is -e_d on the minus face
-      gx += -gla * ds[k * NF + fp_of<N>(0, b, c)] +
-            gra * ds[k * NF + fp_of<N>(1, b, c)];
-      gy += -glb * ds[k * NF + fp_of<N>(2, a, c)] +
-            grb * ds[k * NF + fp_of<N>(3, a, c)];
-      gz += -glc * ds[k * NF + fp_of<N>(4, a, b)] +
-            grc * ds[k * NF + fp_of<N>(5, a, b)];
-      gref[0][k] = gx;
-      gref[1][k] = gy;
-      gref[2][k] = gz;
-    }
-#pragma unroll
-    for (int j = 0; j < 3; ++j)
-#pragma unroll
-      for (int k = 0; k < 5; ++k) {
-        T g = rj * (S[0][j] * gref[0][k] + S[1][j] * gref[1][k] +
-                    S[2][j] * gref[2][k]);
-        grad[(e * 15 + j * 5 + k) * NU + z] = g;
-        gs[(j * 5 + k) * NU + z] = g;
-      }
-  }
-  __syncthreads();
-  if (e >= ne) return;
-  // flux point f with its interpolated gradient g: q (q form) or g itself
-  auto out = [&](int f, const T* g) {
-    if (QV) {
-      T u[5], G[3][5], nv[3], q[5];
-#pragma unroll
-      for (int k = 0; k < 5; ++k) u[k] = ufs[k * NF + f];
-#pragma unroll
-      for (int j = 0; j < 3; ++j) {
-        nv[j] = nvs[j * NF + f];
-#pragma unroll
-        for (int k = 0; k < 5; ++k) G[j][k] = g[j * 5 + k];
-      }
-      visc_q_pre(bc, ph, u, G, nv, int(va.fbc[e * NF + f]), q,
-                 prescribed_at(va, e, f, NF));
-#pragma unroll
-      for (int k = 0; k < 5; ++k) va.q[(e * 5 + k) * NF + f] = q[k];
-    } else {
-#pragma unroll
-      for (int k = 0; k < 15; ++k) va.q[(e * 15 + k) * NF + f] = g[k];
-    }
-  };
-  if constexpr (sizeof(T) == 4) {
-    // shared-memory bound: one thread per face pair (direction, position)
-    for (int t = z; t < 3 * N * N; t += NU) {
-      const int dir = t / (N * N), r = t - dir * N * N, i = r % N, j = r / N;
-      T g0[15], g1[15];
-      face_interp_pair<T, N, 15>(gs, dir, i, j, op, g0, g1);
-      out(fp_of<N>(2 * dir, i, j), g0);
-      out(fp_of<N>(2 * dir + 1, i, j), g1);
-    }
-  } else {
-    // FP64-pipe bound: one thread per flux point spreads the arithmetic
-    for (int f = z; f < NF; f += NU) {
-      T g[15];
-      face_interp<T, N, 15>(gs, f, op, g);
-      out(f, g);
-    }
-  }
-}
-
-// ---------------------------------------------------------------------------
-// Volume kernel on hexahedra: f~ = S F, divergence along the three line
-// families, DG correction with the jump F^C - n~.f~ computed once per flux
-// point, R = -div / J, RK epilogue and the next stage's u_f.
-// Shared memory per element: f~ [3][5][NU] and F^C / jump [5][NF] (type T),
-// then, for FP32 registers, the RK registers X, A [5][NU].  The element's
-// F^C block (and those register blocks) are copied asynchronously
-// (cp.async) at entry, so their loads overlap the flux arithmetic instead
-// of following it.  FP64 registers are read directly: staging them would
-// double the shared memory per element and cost more occupancy than the
-// overlap gains.
-template <typename T, int N>
-__host__ __device__ constexpr int hex_vol_tbytes() {  // T part, 16-byte padded
-  return ((15 * N * N * N + 30 * N * N) * int(sizeof(T)) + 15) / 16 * 16;
-}
-
-template <typename TR>
-__host__ __device__ constexpr bool hex_vol_stage_regs() {
-  return sizeof(TR) == 4;
-}
-
-template <typename T, typename TR, int N>
-__host__ __device__ constexpr int hex_vol_bytes_per_elem() {
-  return hex_vol_tbytes<T, N>() +
-         (hex_vol_stage_regs<TR>() ? (10 * N * N * N * int(sizeof(TR)) + 15) / 16 * 16 : 0);
-}
-
-// AA: f~ is the anti-aliased projection precomputed in tflux
-// ([ne][3][5][NU], Section 3.2) and is copied in instead of collocated.
-template <typename T, typename TR, int N, int EPB, bool NS, bool AA = false>
-__global__ void __launch_bounds__(EPB* N* N* N)
-    k_hex_vol(long long ne, const T* __restrict__ uin, const T* __restrict__ grad,
-              const T* __restrict__ fc, const T* __restrict__ smat,
-              const T* __restrict__ rcpdjac, HexOps<T> op, Phys<T> ph,
-              HexStage<T, TR> sa, const T* __restrict__ tflux = nullptr) {
-  constexpr int NU = N * N * N, NF = 6 * N * N, N2 = N * N;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int le = threadIdx.x / NU, z = threadIdx.x - le * NU;
-  const long long e = (long long)blockIdx.x * (blockDim.x / NU) + le;
-  unsigned char* eb = smem_raw + le * hex_vol_bytes_per_elem<T, TR, N>();
-  T* ft = reinterpret_cast<T*>(eb);       // [3][5][NU]
-  T* jm = ft + 15 * NU;                   // [5][NF]: F^C, then the jump
-  TR* xs = reinterpret_cast<TR*>(eb + hex_vol_tbytes<T, N>());  // [5][NU]
-  TR* as = xs + 5 * NU;                         // [5][NU]
-  const int a = z % N, b = (z / N) % N, c = z / N2;
-  bool nx, na;
-  hex_stage_needs(sa, &nx, &na);
-  constexpr bool SR = hex_vol_stage_regs<TR>();
-  if (e < ne) {
-    async_copy(jm, fc + e * 5 * NF, 5 * NF * int(sizeof(T)), z, NU);
-    if (AA) async_copy(ft, tflux + e * 15 * NU, 15 * NU * int(sizeof(T)), z, NU);
-    if (SR && nx) async_copy(xs, sa.X + e * 5 * NU, 5 * NU * int(sizeof(TR)), z, NU);
-    if (SR && na) async_copy(as, sa.A + e * 5 * NU, 5 * NU * int(sizeof(TR)), z, NU);
-  }
-  T uz[5];
-  if (e < ne) {
-#pragma unroll
-    for (int k = 0; k < 5; ++k)
-      uz[k] = uin ? uin[(e * 5 + k) * NU + z] : T(sa.X[(e * 5 + k) * NU + z]);
-  }
-  if (!AA && e < ne) {
-    T F[3][5];
-    euler_flux(uz, ph, F);
-    if (NS) {
-      T g[3][5];
-#pragma unroll
-      for (int j = 0; j < 3; ++j)
-#pragma unroll
-        for (int k = 0; k < 5; ++k) g[j][k] = grad[(e * 15 + j * 5 + k) * NU + z];
-      viscous_flux_acc(uz, g, ph, T(-1), F);
-    }
-    T S[3][3];
-#pragma unroll
-    for (int r = 0; r < 9; ++r) S[r / 3][r % 3] = smat[(e * 9 + r) * NU + z];
-#pragma unroll
-    for (int d = 0; d < 3; ++d)
-#pragma unroll
-      for (int k = 0; k < 5; ++k)
-        ft[(d * 5 + k) * NU + z] =
-            S[d][0] * F[0][k] + S[d][1] * F[1][k] + S[d][2] * F[2][k];
-  }
-  cp_async_wait_all();
-  __syncthreads();
-  if (e < ne) {
-    // jump at every flux point: F^C - n~ . M0 f~ (only the normal direction,
-    // -e_dir on the minus face, +e_dir on the plus face); FP32: per face
-    // pair (fewer shared reads), FP64: per flux point
-    if constexpr (sizeof(T) == 4) {
-      for (int t = z; t < 3 * N2; t += NU) {
-        const int dir = t / N2, r = t - dir * N2, i = r % N, j = r / N;
-        T f0[5], f1[5];
-        face_interp_pair<T, N, 5>(ft + dir * 5 * NU, dir, i, j, op, f0, f1);
-        const int fm = fp_of<N>(2 * dir, i, j), fp = fp_of<N>(2 * dir + 1, i, j);
-#pragma unroll
-        for (int k = 0; k < 5; ++k) {
-          jm[k * NF + fm] = jm[k * NF + fm] + f0[k];
-          jm[k * NF + fp] = jm[k * NF + fp] - f1[k];
-        }
-      }
-    } else {
-      for (int f = z; f < NF; f += NU) {
-        int face = f / N2;
-        int dir = face >> 1;
-        T fn[5];
-        face_interp<T, N, 5>(ft + dir * 5 * NU, f, op, fn);
-        T sgn = (face & 1) ? T(1) : T(-1);
-#pragma unroll
-        for (int k = 0; k < 5; ++k) jm[k * NF + f] = jm[k * NF + f] - sgn * fn[k];
-      }
-    }
-  }
-  __syncthreads();
-  T s[5];
-  if (e < ne) {
-    T R[5];
-    const T rj = rcpdjac[e * NU + z];
-    T da[N], db[N], dc[N];
-#pragma unroll
-    for (int m = 0; m < N; ++m) {
-      da[m] = op.d1[a][m];
-      db[m] = op.d1[b][m];
-      dc[m] = op.d1[c][m];
-    }
-    const T gla = op.gl[a], gra = op.gr[a], glb = op.gl[b], grb = op.gr[b],
-            glc = op.gl[c], grc = op.gr[c];
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-      const T* fx = ft + (0 * 5 + k) * NU;
-      const T* fy = ft + (1 * 5 + k) * NU;
-      const T* fz = ft + (2 * 5 + k) * NU;
-      T dv = T(0);
-#pragma unroll
-      for (int m = 0; m < N; ++m) {
-        dv += da[m] * fx[m + N * b + N2 * c];
-        dv += db[m] * fy[a + N * m + N2 * c];
-        dv += dc[m] * fz[a + N * b + N2 * m];
-      }
-      const T* jk = jm + k * NF;
-      dv += gla * jk[fp_of<N>(0, b, c)] + gra * jk[fp_of<N>(1, b, c)];
-      dv += glb * jk[fp_of<N>(2, a, c)] + grb * jk[fp_of<N>(3, a, c)];
-      dv += glc * jk[fp_of<N>(4, a, b)] + grc * jk[fp_of<N>(5, a, b)];
-      R[k] = -dv * rj;
-    }
-    TR xr[5], ar[5];
-    if (SR) {
-#pragma unroll
-      for (int k = 0; k < 5; ++k) {
-        xr[k] = nx ? xs[k * NU + z] : TR(0);
-        ar[k] = na ? as[k * NU + z] : TR(0);
-      }
-    } else {
-      hex_stage_load(sa, e * 5 * NU + z, NU, xr, ar);
-    }
-    hex_stage_apply(sa, e * 5 * NU + z, NU, uz, R, xr, ar, s);
-  }
-  if (sa.uf_next == nullptr) return;
-  __syncthreads();
-  if (e < ne) {
-#pragma unroll
-    for (int k = 0; k < 5; ++k) ft[k * NU + z] = s[k];
-  }
-  __syncthreads();
-  if (e >= ne) return;
-  if constexpr (sizeof(T) == 4) {
-    for (int t = z; t < 3 * N2; t += NU) {
-      const int dir = t / N2, r = t - dir * N2, i = r % N, j = r / N;
-      T v0[5], v1[5];
-      face_interp_pair<T, N, 5>(ft, dir, i, j, op, v0, v1);
-      const int fm = fp_of<N>(2 * dir, i, j), fp = fp_of<N>(2 * dir + 1, i, j);
-#pragma unroll
-      for (int k = 0; k < 5; ++k) {
-        sa.uf_next[(e * 5 + k) * NF + fm] = v0[k];
-        sa.uf_next[(e * 5 + k) * NF + fp] = v1[k];
-      }
-    }
-  } else {
-    for (int f = z; f < NF; f += NU) {
-      T v[5];
-      face_interp<T, N, 5>(ft, f, op, v);
-#pragma unroll
-      for (int k = 0; k < 5; ++k) sa.uf_next[(e * 5 + k) * NF + f] = v[k];
     }
   }
 }

@@ -38,7 +38,8 @@
 // coefficients.
 //
 // Measured per launch, 24^3 p = 4 (20^3 p = 3) Navier-Stokes: gradient 850 -> 301
-// us (242 -> 100), volume 1108 -> 268 us (321 -> 95).  What bounds them now:
+// us (242 -> 100; 344 with the solution jumps taken in the kernel, which
+// saves the 43 us of a kernel for them), volume 1108 -> 268 us (321 -> 95).  What bounds them now:
 // the ALU pipe and the FP64 pipe are each at 48-59 %, the rest is the latency
 // of dependent integer instructions at 24 warps per SM (80 registers; 64
 // spill, 96 leave fewer warps, both slower).
@@ -328,7 +329,7 @@ __host__ __device__ constexpr int hexfx_bytes_per_elem(bool grad) {
   return (slots * 8 + (G::WPE * 6 + 16 + 8) * 4 + 15) / 16 * 16;
 }
 
-// NS gradients (as k_hex_grad with QV = false): corrected reference gradient
+// NS gradients: corrected reference gradient
 // by lines, physical gradient by the fixed-point S / det J, its 15 components
 // at the flux points by lines.  At the solution points the volume kernel
 // needs the viscous flux alone: it is formed here, where the FP64 pipe is
@@ -336,8 +337,9 @@ __host__ __device__ constexpr int hexfx_bytes_per_elem(bool grad) {
 // gradient components would also be 6 more to write and read).  RAW: the
 // gradient itself [ne][15][nu], for the anti-aliased flux.
 template <int N, int EPB, bool RAW>
-__global__ void __launch_bounds__(EPB* FxGeom<N>::TPE, 3)
-    k_hexfx_grad(long long ne, const double* __restrict__ u, const double* __restrict__ du,
+__global__ void __launch_bounds__(EPB* FxGeom<N>::TPE, N == 3 ? 2 : 3)
+    k_hexfx_grad(long long ne, const double* __restrict__ u,
+                 const __grid_constant__ TraceArgs<double> ta,
                  const FxCoef* __restrict__ jq, const int* __restrict__ jex,
                  const __grid_constant__ HexFxOps op, Phys<double> ph,
                  double* __restrict__ grad, double* __restrict__ gradf) {
@@ -368,12 +370,14 @@ __global__ void __launch_bounds__(EPB* FxGeom<N>::TPE, 3)
       mx[k] = fx_mag(uv[k]);
     }
 #pragma unroll
-    for (int i = 0; i < NFT; ++i)
+    for (int i = 0; i < NFT; ++i) {
+      if (z + i * TPE < NF) {
+        double own[5];
+        trace_jump(ta, e, z + i * TPE, NF, own, dv[i]);
 #pragma unroll
-      for (int k = 0; k < 5; ++k) {
-        dv[i][k] = z + i * TPE < NF ? du[(e * 5 + k) * NF + z + i * TPE] : 0.0;
-        mx[k] = max(mx[k], fx_mag(dv[i][k]));
+        for (int k = 0; k < 5; ++k) mx[k] = max(mx[k], fx_mag(dv[i][k]));
       }
+    }
     fx_warp_max<5>(mx, ex, wz);
     fx_sync<G::WPE, EPB>(le);
 #pragma unroll
@@ -510,13 +514,13 @@ __global__ void __launch_bounds__(EPB* FxGeom<N>::TPE, 3)
   }
 }
 
-// Volume kernel (as k_hex_vol): flux in FP64, f~ = S F, jump, divergence and
+// Volume kernel: flux in FP64, f~ = S F, jump, divergence and
 // correction in fixed point, R = -div / J and the RK epilogue in FP64, the
 // next stage's u_f by lines in fixed point.  The three momentum variables
 // share one field exponent (their flux tensor is symmetric).  visc: the
 // viscous flux of k_hexfx_grad.
 template <int N, int EPB, bool NS, bool AA = false>
-__global__ void __launch_bounds__(EPB* FxGeom<N>::TPE, 3)
+__global__ void __launch_bounds__(EPB* FxGeom<N>::TPE, N == 3 ? 2 : 3)
     k_hexfx_vol(long long ne, const double* __restrict__ u, const double* __restrict__ visc,
                 const double* __restrict__ fc, const FxCoef* __restrict__ sq,
                 const int* __restrict__ sex, const double* __restrict__ rcpdjac,

@@ -19,6 +19,12 @@
 // separate kernel would write, and stores the viscous flux at the solution
 // points (9 values) in place of the gradient (15): together 12 KB of 59 KB
 // DRAM traffic an element and stage less at p = 4.
+//
+// Measured per launch, 48^3 p = 4 with FP64 registers (32^3 p = 3 FP32):
+// common solution and gradient 155 + 621 -> 586 us (29 + 85 -> 96), volume 657 ->
+// 550-583 us (92 -> 71; 0.9 of its DRAM traffic at the copy rate).  The
+// gradient kernel issues on 65 % of the cycles and waits for the traces on
+// most of the others.
 #pragma once
 #include "fr_hexfx.cuh"
 
@@ -43,14 +49,24 @@ __host__ __device__ constexpr int hexl_vol_bytes() {
   return (15 * G::PN + 5 * G::NF) * int(sizeof(T));
 }
 
-// the line of task r (0 .. 3 N^2 - 1): direction, first slot, stride, minus
-// face flux point
+// Lines of a CTA, numbered direction by direction (for N = 4 and an even
+// number of elements a warp's 32 lines then run the same way, on distinct
+// banks; padding the directions to whole warps for the other N was slower).
 template <int N>
-__device__ __forceinline__ int hexl_line(int r, int* s0, int* st, int* fm) {
-  const int d = r / (N * N);
-  fx_line<N>(d, r - d * N * N, s0, st, fm);
-  return d;
-}
+struct LineTasks {
+  int per, lines;  // slots and real lines of a direction
+  __device__ __forceinline__ LineTasks(int eb, int nel) : per(eb * N * N), lines(nel * N * N) {}
+  __device__ __forceinline__ int count() const { return 3 * per; }
+  // element, direction, first slot, stride and minus-face flux point of line
+  // t; false: no element there (a ragged last CTA)
+  __device__ __forceinline__ bool get(int t, int* le, int* d, int* s0, int* st, int* fm) const {
+    *d = (t >= per) + (t >= 2 * per);
+    const int r = t - *d * per;
+    *le = r / (N * N);
+    fx_line<N>(*d, r - *le * N * N, s0, st, fm);
+    return r < lines;
+  }
+};
 
 // values at a line's two faces (Gauss-Lobatto: the line's end points)
 template <typename T, int N>
@@ -74,10 +90,11 @@ __device__ __forceinline__ void hexl_faces(const HexOps<T>& op, const T v[N], T*
 // mass component is zero and stays as allocated); FP64: the 15 gradient
 // components there.  At the solution points the viscous flux [ne][9][nu]; RAW:
 // the gradient [ne][15][nu] (anti-aliased flux).
+// FP32: 64 registers (1024 threads per SM; 48 spill, 80 are slower).
 template <typename T, typename TR, int N, int EPB, bool RAW>
-__global__ void __launch_bounds__(hexl_threads<N>(EPB))
+__global__ void __launch_bounds__(hexl_threads<N>(EPB), sizeof(T) == 4 ? 4 : 2)
     k_hexl_grad(long long ne, int eb, const T* __restrict__ uin, const TR* __restrict__ X,
-                TraceArgs<T> ta, const T* __restrict__ smat, const T* __restrict__ rcpdjac,
+                const __grid_constant__ TraceArgs<T> ta, const T* __restrict__ smat, const T* __restrict__ rcpdjac,
                 const __grid_constant__ HexOps<T> op, T* __restrict__ grad, ViscArgs<T> va,
                 const __grid_constant__ BCTab<T> bc, Phys<T> ph) {
   using G = FxGeom<N>;
@@ -86,6 +103,7 @@ __global__ void __launch_bounds__(hexl_threads<N>(EPB))
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const long long e0 = (long long)blockIdx.x * eb;
   const int nel = int(ne - e0 < eb ? ne - e0 : eb);
+  const LineTasks<N> lines(eb, nel);
   T* us = reinterpret_cast<T*>(smem_raw);  // [eb][5][PN]
   T* ds = us + eb * 5 * PN;                // [eb][5][NF]
   T* gs = ds + eb * 5 * NF;                // [eb][15][PN]
@@ -94,35 +112,50 @@ __global__ void __launch_bounds__(hexl_threads<N>(EPB))
   const bool pt = le < nel;
   const long long e = e0 + le;
   const int slot = G::slot(z % N, (z / N) % N, z / N2);
+  // all loads first, the partner codes before everything else: their values
+  // address the partners' traces
+  constexpr int NT = (NF + NU - 1) / NU;
+  TraceSide<T> side[NT];
+  T own[NT][5], jmp[NT][5], uv[5], S[9], rj = T(0);
+#pragma unroll
+  for (int i = 0; i < NT; ++i) {
+    const int t = threadIdx.x + i * blockDim.x;
+    if (t < nel * NF) side[i].init(ta, e0 + t / NF, t % NF, NF);
+  }
+#pragma unroll
+  for (int i = 0; i < NT; ++i) {
+    const int t = threadIdx.x + i * blockDim.x;
+    if (t < nel * NF) side[i].load(ta, e0 + t / NF, t % NF, NF, own[i], jmp[i]);
+  }
   if (pt) {
 #pragma unroll
     for (int k = 0; k < 5; ++k)
-      us[(le * 5 + k) * PN + slot] =
-          uin ? uin[(e * 5 + k) * NU + z] : T(X[(e * 5 + k) * NU + z]);
-  }
-  for (int t = threadIdx.x; t < nel * NF; t += blockDim.x) {
-    const int l = t / NF, f = t - l * NF;
-    T own[5], d[5];
-    trace_jump(ta, e0 + l, f, NF, own, d);
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-      ds[(l * 5 + k) * NF + f] = d[k];
-      if (QV) fs[(l * 5 + k) * NF + f] = own[k];
-    }
-  }
-  T S[9], rj = T(0);
-  if (pt) {  // read ahead of the line phase
+      uv[k] = uin ? uin[(e * 5 + k) * NU + z] : T(X[(e * 5 + k) * NU + z]);
 #pragma unroll
     for (int r = 0; r < 9; ++r) S[r] = smat[(e * 9 + r) * NU + z];
     rj = rcpdjac[e * NU + z];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) us[(le * 5 + k) * PN + slot] = uv[k];
+  }
+#pragma unroll
+  for (int i = 0; i < NT; ++i) {
+    const int t = threadIdx.x + i * blockDim.x;
+    if (t < nel * NF) {
+      const int l = t / NF, f = t - l * NF;
+      side[i].jump(own[i], jmp[i]);
+#pragma unroll
+      for (int k = 0; k < 5; ++k) {
+        ds[(l * 5 + k) * NF + f] = jmp[i][k];
+        if (QV) fs[(l * 5 + k) * NF + f] = own[i][k];
+      }
+    }
   }
   __syncthreads();
   // reference gradient along every line, with the correction of the jumps
   // (the face normal is -e_d on the minus face)
-  for (int t = threadIdx.x; t < nel * 3 * N2; t += blockDim.x) {
-    const int l = t / (3 * N2);
-    int s0, st, fm;
-    const int d = hexl_line<N>(t - l * 3 * N2, &s0, &st, &fm);
+  for (int t = threadIdx.x; t < lines.count(); t += blockDim.x) {
+    int l, d, s0, st, fm;
+    if (!lines.get(t, &l, &d, &s0, &st, &fm)) continue;
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
       const T* p = us + (l * 5 + k) * PN + s0;
@@ -166,11 +199,10 @@ __global__ void __launch_bounds__(hexl_threads<N>(EPB))
     }
   }
   __syncthreads();
-  for (int t = threadIdx.x; t < nel * 3 * N2; t += blockDim.x) {
-    const int l = t / (3 * N2);
+  for (int t = threadIdx.x; t < lines.count(); t += blockDim.x) {
+    int l, d, s0, st, fm;
+    if (!lines.get(t, &l, &d, &s0, &st, &fm)) continue;
     const long long el = e0 + l;
-    int s0, st, fm;
-    hexl_line<N>(t - l * 3 * N2, &s0, &st, &fm);
     const T* p = gs + l * 15 * PN + s0;
     T g0[3][5], g1[3][5];
 #pragma unroll
@@ -206,7 +238,7 @@ __global__ void __launch_bounds__(hexl_threads<N>(EPB))
 // line's f~), R = -div / J, the RK epilogue and the next stage's u_f.  visc:
 // the viscous flux of k_hexl_grad; AA: f~ comes projected in tflux.
 template <typename T, typename TR, int N, int EPB, bool NS, bool AA = false>
-__global__ void __launch_bounds__(hexl_threads<N>(EPB))
+__global__ void __launch_bounds__(hexl_threads<N>(EPB), sizeof(T) == 4 ? 5 : 2)
     k_hexl_vol(long long ne, int eb, const T* __restrict__ uin, const T* __restrict__ visc,
                const T* __restrict__ fc, const T* __restrict__ smat,
                const T* __restrict__ rcpdjac, const __grid_constant__ HexOps<T> op, Phys<T> ph,
@@ -216,6 +248,7 @@ __global__ void __launch_bounds__(hexl_threads<N>(EPB))
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const long long e0 = (long long)blockIdx.x * eb;
   const int nel = int(ne - e0 < eb ? ne - e0 : eb);
+  const LineTasks<N> lines(eb, nel);
   T* ft = reinterpret_cast<T*>(smem_raw);  // [eb][15][PN]
   T* cs = ft + eb * 15 * PN;               // [eb][5][NF]
   const int le = threadIdx.x / NU, z = threadIdx.x - le * NU;
@@ -258,10 +291,9 @@ __global__ void __launch_bounds__(hexl_threads<N>(EPB))
     hex_stage_load(sa, e * 5 * NU + z, NU, xr, ar);
     rj = rcpdjac[e * NU + z];
   }
-  for (int t = threadIdx.x; t < nel * 3 * N2; t += blockDim.x) {
-    const int l = t / (3 * N2);
-    int s0, st, fm;
-    const int d = hexl_line<N>(t - l * 3 * N2, &s0, &st, &fm);
+  for (int t = threadIdx.x; t < lines.count(); t += blockDim.x) {
+    int l, d, s0, st, fm;
+    if (!lines.get(t, &l, &d, &s0, &st, &fm)) continue;
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
       T* p = ft + (l * 15 + d * 5 + k) * PN + s0;
@@ -292,10 +324,9 @@ __global__ void __launch_bounds__(hexl_threads<N>(EPB))
   }
   if (sa.uf_next == nullptr) return;
   __syncthreads();
-  for (int t = threadIdx.x; t < nel * 3 * N2; t += blockDim.x) {
-    const int l = t / (3 * N2);
-    int s0, st, fm;
-    hexl_line<N>(t - l * 3 * N2, &s0, &st, &fm);
+  for (int t = threadIdx.x; t < lines.count(); t += blockDim.x) {
+    int l, d, s0, st, fm;
+    if (!lines.get(t, &l, &d, &s0, &st, &fm)) continue;
     T* o = sa.uf_next + (e0 + l) * 5 * NF + fm;
 #pragma unroll
     for (int k = 0; k < 5; ++k) {

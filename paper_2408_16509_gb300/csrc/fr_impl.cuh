@@ -25,6 +25,7 @@
 #include "fr_filter.cuh"
 #include "fr_hex.cuh"
 #include "fr_hexfx.cuh"
+#include "fr_hexline.cuh"
 #include "fr_kernels.cuh"
 #include "fr_prism.cuh"
 #include "fr_err.hpp"
@@ -87,6 +88,9 @@ struct DevType {
   int kind = 0, nu = 0, nf = 0;
   long long ne = 0;
   long long off_f = 0;      // offset of this type in the flux-point buffers
+  int tidx = 0;             // index of the type in the mesh
+  long long e0 = 0;         // first element (a sub-range of a type)
+  int32_t* fpartner = nullptr;  // [ne][nf] partner flux-point code, -1: boundary
   void* X = nullptr;        // solution register        [ne][5][nu]
   void* Y = nullptr;        // stage register
   void* A = nullptr;        // RK4 accumulator
@@ -112,7 +116,6 @@ struct DevType {
   void* fVT = nullptr;
   void* fdeg = nullptr;
   void* fW = nullptr;
-  int32_t* fpartner = nullptr;
   int32_t* flist = nullptr;  // [ne] elements that fail the zeta = 0 test
   int* fcount = nullptr;     // their number
   double* smin = nullptr;
@@ -596,6 +599,45 @@ constexpr bool tc_types() {
   return std::is_same<T, float>::value && std::is_same<TR, float>::value;
 }
 
+// Partner code of every flux point (-1 on boundaries): both sides of a pair
+// name each other.
+static __global__ void k_partner(int np, const int32_t* __restrict__ pl,
+                                 const int32_t* __restrict__ pr, int32_t* t0, int32_t* t1,
+                                 int32_t* t2, int nf0, int nf1, int nf2) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= np) return;
+  auto put = [&](int32_t at, int32_t code) {
+    const int t = at >> 29;
+    const unsigned l = unsigned(at) & ((1u << 29) - 1);
+    const unsigned nf = unsigned(t == 0 ? nf0 : t == 1 ? nf1 : nf2);
+    int32_t* p = t == 0 ? t0 : t == 1 ? t1 : t2;
+    p[(long long)(l / (5 * nf)) * nf + l % nf] = code;
+  };
+  put(pl[i], pr[i]);
+  put(pr[i], pl[i]);
+}
+
+inline int setup_partner(fr_mesh* m) {
+  int32_t* p[3] = {nullptr, nullptr, nullptr};
+  int nf[3] = {1, 1, 1};
+  for (size_t t = 0; t < m->types.size(); ++t) {
+    DevType& D = m->types[t];
+    if (D.fpartner) return FR_OK;
+    const size_t bytes = size_t(D.ne) * D.nf * sizeof(int32_t);
+    CK(cudaMalloc((void**)&D.fpartner, bytes));
+    m->allocs.push_back(D.fpartner);
+    CK(cudaMemset(D.fpartner, 0xff, bytes));
+    p[t] = D.fpartner;
+    nf[t] = D.nf;
+  }
+  if (m->np)
+    k_partner<<<unsigned((m->np + 255) / 256), 256>>>(m->np, m->pl, m->pr, p[0], p[1], p[2],
+                                                       nf[0], nf[1], nf[2]);
+  CK(cudaGetLastError());
+  CK(cudaDeviceSynchronize());
+  return FR_OK;
+}
+
 // T: storage/compute type of traces, fluxes and stage values;
 // TR: type of the RK solution and accumulator registers (X, A).
 template <typename T, typename TR>
@@ -606,6 +648,7 @@ int setup_device(fr_mesh* m) {
     const HostType& H = m->host[t];
     DevType D;
     D.kind = H.kind;
+    D.tidx = int(t);
     D.curved = H.map_order >= 2;
     D.nu = H.ref.nupts;
     D.nf = H.ref.nfpts;
@@ -797,6 +840,7 @@ int setup_device(fr_mesh* m) {
   if ((rc = dev_upload_i32(m, C.pr, &m->pr))) return rc;
   if ((rc = dev_upload<T>(m, C.pn, &m->pn))) return rc;
   if ((rc = dev_upload<T>(m, C.pmr, &m->pmr))) return rc;
+  if (m->physics == FR_NAVIER_STOKES && (rc = setup_partner(m))) return rc;
   if ((rc = dev_upload_i32(m, C.bidx, &m->bidx))) return rc;
   if ((rc = dev_upload_i32(m, C.bbc, &m->bbc))) return rc;
   if ((rc = dev_upload<T>(m, C.bn, &m->bn))) return rc;
@@ -881,16 +925,6 @@ bool hex_dispatch(int p, F&& f) {
 template <int N>
 constexpr int hex_epb() {
   return (N * N * N) >= 256 ? 1 : 256 / (N * N * N);
-}
-
-template <typename T, typename TR, int N>
-constexpr size_t hex_vol_smem() {
-  return size_t(hex_epb<N>()) * size_t(hex_vol_bytes_per_elem<T, TR, N>());
-}
-
-template <typename T, int N>
-constexpr size_t hex_grad_smem() {
-  return size_t(hex_epb<N>()) * size_t(hex_grad_bytes_per_elem<T, N, sizeof(T) == 4>());
 }
 
 bool use_hex(const fr_mesh* m, const DevType& D) {
@@ -1170,13 +1204,12 @@ int prepare_kernels(fr_mesh* m) {
                         k_hexfx_vol<N, E, false, true>})
           cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, sv);
       } else {
-        const int sv = int(hex_vol_smem<T, TR, N>());
-        for (auto fn : {k_hex_vol<T, TR, N, E, false>, k_hex_vol<T, TR, N, E, true>,
-                        k_hex_vol<T, TR, N, E, false, true>, k_hex_vol<T, TR, N, E, true, true>})
+        const int sg = E * hexl_grad_bytes<T, N>(), sv = E * hexl_vol_bytes<T, N>();
+        for (auto fn : {k_hexl_grad<T, TR, N, E, false>, k_hexl_grad<T, TR, N, E, true>})
+          cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, sg);
+        for (auto fn : {k_hexl_vol<T, TR, N, E, false>, k_hexl_vol<T, TR, N, E, true>,
+                        k_hexl_vol<T, TR, N, E, false, true>})
           cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, sv);
-        cudaFuncSetAttribute(k_hex_grad<T, TR, N, E, sizeof(T) == 4>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             int(hex_grad_smem<T, N>()));
         cudaFuncSetAttribute(k_hex_grad_v<T, TR, N, E>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize,
                              int(hexv_grad_smem<T, N>()));
@@ -1281,6 +1314,7 @@ inline std::vector<int> tile_candidates(const fr_mesh* m, const DevType& D, bool
 inline DevType sub_view(const fr_mesh* m, const DevType& D, long long e0, long long n) {
   DevType V = D;
   V.ne = n;
+  V.e0 = D.e0 + e0;
   const size_t w = m->wsize, r = m->rsize, nu = size_t(D.nu), nf = size_t(D.nf);
   auto sh = [&](void* p, size_t per) -> void* {
     return p ? static_cast<void*>(static_cast<char*>(p) + size_t(e0) * per) : nullptr;
@@ -1300,6 +1334,7 @@ inline DevType sub_view(const fr_mesh* m, const DevType& D, long long e0, long l
   V.fnv = sh(D.fnv, 3 * nf * w);
   V.fbc = static_cast<int8_t*>(sh(D.fbc, nf));
   V.fbi = static_cast<int32_t*>(sh(D.fbi, nf * sizeof(int32_t)));
+  V.fpartner = static_cast<int32_t*>(sh(D.fpartner, nf * sizeof(int32_t)));
   V.verts = sh(D.verts, 24 * w);
   V.aasmq = sh(D.aasmq, 9 * size_t(D.aa_nq) * w);
   V.tf = sh(D.tf, 15 * nu * w);
@@ -1374,7 +1409,14 @@ void launch_stage(fr_mesh* m, cudaStream_t s, int mode, int stage,
     PROF_END(FR_KC_FILTER);
   }
   if (ns && (phase & 1)) {
-    if (m->np && pairs) {
+    // the jumps of interior points: the gradient kernels take them from the
+    // traces themselves, except the vertex-metric family (its volume kernel
+    // needs them again after the traces have moved on) and the tensor cores
+    bool need_du = false;
+    for (auto& D : m->types)
+      need_du |= use_tc_grad(m, D) ||
+                 (use_hex(m, D) && D.verts && m->active == FR_VARIANT_SUMFACT_VERTEX);
+    if (m->np && pairs && need_du) {
       PROF_BEGIN(FR_KC_FACE_U);
       k_face_ucommon<T><<<nblk(m->np, tb), tb, 0, s>>>(
           m->np, m->pl, m->pr, (const T*)m->uf, (T*)m->du, m->tt, ph.beta);
@@ -1392,6 +1434,9 @@ void launch_stage(fr_mesh* m, cudaStream_t s, int mode, int stage,
                      (T*)m->gradf + D.off_f * (sizeof(T) == 4 ? 1 : 3)};
       va.fbi = D.fbi;
       va.xp = (const T*)m->xu;
+      const TraceArgs<T> ta{va.uf, (const T*)m->uf, du, D.fpartner, m->tt,
+                            ((long long)D.tidx << 29) + D.e0 * 5 * D.nf,
+                            T(0.5) + ph.beta, T(0.5) - ph.beta};
       PROF_BEGIN(FR_KC_GRAD);
       if (use_hex(m, D) && sizeof(T) == 4 && D.verts &&
           m->active == FR_VARIANT_SUMFACT_VERTEX) {
@@ -1414,17 +1459,24 @@ void launch_stage(fr_mesh* m, cudaStream_t s, int mode, int stage,
             const size_t sm = size_t(eb) * hexfx_bytes_per_elem<N>(true);
             const T* uin = from_x ? (const T*)D.X : (const T*)D.Y;
             if (m->aa_qdeg > 0)
-              k_hexfx_grad<N, E, true><<<grid, tpb, sm, s>>>(D.ne, uin, du, D.fxj, D.fxe, D.hxfx,
+              k_hexfx_grad<N, E, true><<<grid, tpb, sm, s>>>(D.ne, uin, ta, D.fxj, D.fxe, D.hxfx,
                                                              ph, (T*)D.grad, va.q);
             else
-              k_hexfx_grad<N, E, false><<<grid, tpb, sm, s>>>(D.ne, uin, du, D.fxj, D.fxe, D.hxfx,
+              k_hexfx_grad<N, E, false><<<grid, tpb, sm, s>>>(D.ne, uin, ta, D.fxj, D.fxe, D.hxfx,
                                                               ph, (T*)D.grad, va.q);
-          } else
-            k_hex_grad<T, TR, N, E, sizeof(T) == 4>
-                <<<nblk(D.ne, eb), eb * N * N * N, hex_grad_smem<T, N>() / E * eb, s>>>(
-                    D.ne, from_x ? nullptr : (const T*)D.Y, (const TR*)D.X, du,
-                    (const T*)D.smat, (const T*)D.rcpdjac, hexops<T>(D),
-                    (T*)D.grad, va, bc, ph);
+          } else {
+            const unsigned grid = nblk(D.ne, eb), tpb = hexl_threads<N>(eb);
+            const size_t sm = size_t(eb) * hexl_grad_bytes<T, N>();
+            const T* uin = from_x ? nullptr : (const T*)D.Y;
+            if (m->aa_qdeg > 0)
+              k_hexl_grad<T, TR, N, E, true><<<grid, tpb, sm, s>>>(
+                  D.ne, eb, uin, (const TR*)D.X, ta, (const T*)D.smat, (const T*)D.rcpdjac,
+                  hexops<T>(D), (T*)D.grad, va, bc, ph);
+            else
+              k_hexl_grad<T, TR, N, E, false><<<grid, tpb, sm, s>>>(
+                  D.ne, eb, uin, (const TR*)D.X, ta, (const T*)D.smat, (const T*)D.rcpdjac,
+                  hexops<T>(D), (T*)D.grad, va, bc, ph);
+          }
         });
       } else if (use_tc_grad(m, D)) {
         launch_grad_tc<T, TR>(m, D, s, from_x, du, va, bc, ph);
@@ -1438,7 +1490,7 @@ void launch_stage(fr_mesh* m, cudaStream_t s, int mode, int stage,
                 (long long)m->num_sms * (D.tile_grad > 0 ? D.tile_grad : D.pri_grad_ctas)));
             k_grad_pri<T, NU, NF, E, sizeof(T) == 4>
                 <<<grid, E * NU, pri_grad_smem<T, NU, NF>(D), s>>>(
-                    D.ne, from_x ? (const T*)D.X : (const T*)D.Y, du, (const T*)D.smat,
+                    D.ne, from_x ? (const T*)D.X : (const T*)D.Y, ta, (const T*)D.smat,
                     (const T*)D.rcpdjac, pri_ops_of<T>(m, D), (T*)D.grad, va, bc, ph);
           }
         });
@@ -1451,7 +1503,7 @@ void launch_stage(fr_mesh* m, cudaStream_t s, int mode, int stage,
               (D.ne + E - 1) / E,
               (long long)m->num_sms * (D.tile_grad > 0 ? D.tile_grad : D.grad_ctas)));
           k_grad_dense<T, NU, NF, E, sizeof(T) == 4><<<grid, E * NU, sm, s>>>(
-              D.ne, from_x ? (const T*)D.X : (const T*)D.Y, du,
+              D.ne, from_x ? (const T*)D.X : (const T*)D.Y, ta,
               (const T*)D.smat, (const T*)D.rcpdjac, stage_ops_of<T>(m, D), (T*)D.grad,
               va, bc, ph);
         });
@@ -1526,7 +1578,8 @@ void launch_stage(fr_mesh* m, cudaStream_t s, int mode, int stage,
             k_hexfx_vol<N, E, false><<<grid, tpb, sm, s>>>(
                 D.ne, uin, nullptr, fc, D.fxs, D.fxe, (const T*)D.rcpdjac, D.hxfx, ph, sa);
         } else {
-          const size_t sm = hex_vol_smem<T, TR, N>() / E * eb;
+          const size_t sm = size_t(eb) * hexl_vol_bytes<T, N>();
+          const unsigned grid = nblk(D.ne, eb), tpb = hexl_threads<N>(eb);
           const T* uin = from_x ? nullptr : (const T*)D.Y;
           if (sizeof(T) == 4 && D.verts && m->active == FR_VARIANT_SUMFACT_VERTEX) {
             const size_t smv = hexv_vol_smem<T, TR, N>() / E * eb;
@@ -1539,21 +1592,17 @@ void launch_stage(fr_mesh* m, cudaStream_t s, int mode, int stage,
                   D.ne, uin, nullptr, fc, (const T*)D.verts, hexops<T>(D), ph, sa);
             return;
           }
-          if (aa && ns)
-            k_hex_vol<T, TR, N, E, true, true><<<nblk(D.ne, eb), eb * N * N * N, sm, s>>>(
-                D.ne, uin, nullptr, fc, nullptr, (const T*)D.rcpdjac, hexops<T>(D),
-                ph, sa, (const T*)D.tf);
-          else if (aa)
-            k_hex_vol<T, TR, N, E, false, true><<<nblk(D.ne, eb), eb * N * N * N, sm, s>>>(
-                D.ne, uin, nullptr, fc, nullptr, (const T*)D.rcpdjac, hexops<T>(D),
-                ph, sa, (const T*)D.tf);
+          if (aa)
+            k_hexl_vol<T, TR, N, E, false, true><<<grid, tpb, sm, s>>>(
+                D.ne, eb, uin, nullptr, fc, nullptr, (const T*)D.rcpdjac, hexops<T>(D), ph, sa,
+                (const T*)D.tf);
           else if (ns)
-            k_hex_vol<T, TR, N, E, true><<<nblk(D.ne, eb), eb * N * N * N, sm, s>>>(
-                D.ne, uin, (const T*)D.grad, fc, (const T*)D.smat,
-                (const T*)D.rcpdjac, hexops<T>(D), ph, sa);
+            k_hexl_vol<T, TR, N, E, true><<<grid, tpb, sm, s>>>(
+                D.ne, eb, uin, (const T*)D.grad, fc, (const T*)D.smat, (const T*)D.rcpdjac,
+                hexops<T>(D), ph, sa);
           else
-            k_hex_vol<T, TR, N, E, false><<<nblk(D.ne, eb), eb * N * N * N, sm, s>>>(
-                D.ne, uin, nullptr, fc, (const T*)D.smat, (const T*)D.rcpdjac,
+            k_hexl_vol<T, TR, N, E, false><<<grid, tpb, sm, s>>>(
+                D.ne, eb, uin, nullptr, fc, (const T*)D.smat, (const T*)D.rcpdjac,
                 hexops<T>(D), ph, sa);
         }
       });

@@ -457,6 +457,66 @@ __device__ __forceinline__ void write_visc_q(const ViscArgs<T>& va,
   for (int k = 0; k < 5; ++k) va.q[(e * 5 + k) * nf + f] = q[k];
 }
 
+// Traces on both sides of an element type's flux points.
+template <typename T>
+struct TraceArgs {
+  const T* uf;               // this type's [ne][5][nf] traces
+  const T* uf_all;           // all types' traces
+  const T* du;               // this type's [ne][5][nf] jumps (boundary points)
+  const int32_t* partner;    // this type's [ne][nf]: partner code, -1: boundary
+  TypeTab tt;
+  long long code0;           // code of flux point 0 of element 0
+  T wl, wr;                  // u^C - u = w (partner - own): the "-" / "+" side
+};
+
+// The other side of a flux point: the partner's trace with the weight of this
+// side, or on a boundary the stored jump (weight 1, nothing subtracted).
+template <typename T>
+struct TraceSide {
+  const T* p;
+  long long stride;
+  T w;
+  bool interior;
+  __device__ __forceinline__ void init(const TraceArgs<T>& ta, long long e, int f, int nf) {
+    const int32_t c = ta.partner[e * nf + f];
+    interior = c >= 0;
+    if (interior) {
+      const FluxPt q(c, ta.tt);
+      p = ta.uf_all + q.p5;
+      stride = q.nf;
+      // the "-" side is the one with the lower code (type, element, face)
+      w = ta.code0 + e * 5 * nf + f < (long long)c ? ta.wl : ta.wr;
+    } else {
+      p = ta.du + e * 5 * nf + f;
+      stride = nf;
+      w = T(1);
+    }
+  }
+  __device__ __forceinline__ void load(const TraceArgs<T>& ta, long long e, int f, int nf,
+                                       T own[5], T other[5]) const {
+    const T* po = ta.uf + e * 5 * nf + f;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) own[k] = po[k * nf];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) other[k] = p[k * stride];
+  }
+  // other -> u^C - own
+  __device__ __forceinline__ void jump(const T own[5], T other[5]) const {
+#pragma unroll
+    for (int k = 0; k < 5; ++k) other[k] = w * (interior ? other[k] - own[k] : other[k]);
+  }
+};
+
+// own[5]: the element's trace at flux point f; d[5]: u^C - own
+template <typename T>
+__device__ __forceinline__ void trace_jump(const TraceArgs<T>& ta, long long e, int f, int nf,
+                                           T own[5], T d[5]) {
+  TraceSide<T> s;
+  s.init(ta, e, f, nf);
+  s.load(ta, e, f, nf, own, d);
+  s.jump(own, d);
+}
+
 // Viscous normal flux q of write_visc_q from inputs read beforehand: u
 // (trace), G (gradient at the flux point), nv = S^T n~, b = boundary-
 // condition index or -1.
@@ -507,8 +567,8 @@ __global__ void k_face_flux_ns(int np, const int32_t* __restrict__ pl,
     const long long il = L.p5 + (long long)k * L.nf, ir = R.p5 + (long long)k * R.nf;
     ul[k] = uf[il];
     ur[k] = uf[ir];
-    ql[k] = q[il];
-    qr[k] = q[ir];
+    ql[k] = k ? q[il] : T(0);  // no viscous mass flux
+    qr[k] = k ? q[ir] : T(0);
   }
   T n[3] = {pn[4 * i], pn[4 * i + 1], pn[4 * i + 2]};
   T ml = pn[4 * i + 3], mr = pmr[i];
@@ -764,7 +824,7 @@ __device__ __forceinline__ DenseOps<T> stage_dense_ops(const DenseOps<T>& g,
 template <typename T, int NU, int NF, int EPB, bool QV>
 __global__ void __launch_bounds__(EPB* NU)
     k_grad_dense(long long ne, const T* __restrict__ u,
-                 const T* __restrict__ du, const T* __restrict__ smat,
+                 const __grid_constant__ TraceArgs<T> ta, const T* __restrict__ smat,
                  const T* __restrict__ rcpdjac, DenseOps<T> gops,
                  T* __restrict__ grad, ViscArgs<T> va, BCTab<T> bc,
                  Phys<T> ph) {
@@ -788,8 +848,8 @@ __global__ void __launch_bounds__(EPB* NU)
       for (int k = 0; k < 5; ++k) v[k] = u[(e * 5 + k) * NU + z];
       put5<L, NU>(us, z, v);
       for (int f = z; f < NF; f += NU) {
-#pragma unroll
-        for (int k = 0; k < 5; ++k) v[k] = du[(e * 5 + k) * NF + f];
+        T own[5];
+        trace_jump(ta, e, f, NF, own, v);
         put5<L, NF>(ds, f, v);
       }
     }

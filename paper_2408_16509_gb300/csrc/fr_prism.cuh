@@ -101,7 +101,8 @@ __device__ __forceinline__ PriOps<T> stage_pri_ops(const PriOps<T>& g, unsigned 
 // its values at the flux points (q form: the viscous normal flux there).
 template <typename T, int NU, int NF, int EPB, bool QV>
 __global__ void __launch_bounds__(EPB* NU)
-    k_grad_pri(long long ne, const T* __restrict__ u, const T* __restrict__ du,
+    k_grad_pri(long long ne, const T* __restrict__ u,
+               const __grid_constant__ TraceArgs<T> ta,
                const T* __restrict__ smat, const T* __restrict__ rcpdjac, PriOps<T> gops,
                T* __restrict__ grad, ViscArgs<T> va, BCTab<T> bc, Phys<T> ph) {
   using L = DenseLayout<T, NU, NF>;
@@ -125,8 +126,8 @@ __global__ void __launch_bounds__(EPB* NU)
       for (int k = 0; k < 5; ++k) v[k] = u[(e * 5 + k) * NU + z];
       put5<L, NU>(us, z, v);
       for (int f = z; f < NF; f += NU) {
-#pragma unroll
-        for (int k = 0; k < 5; ++k) v[k] = du[(e * 5 + k) * NF + f];
+        T own[5];
+        trace_jump(ta, e, f, NF, own, v);
         put5<L, NF>(ds, f, v);
       }
     }
