@@ -931,6 +931,12 @@ bool use_hex(const fr_mesh* m, const DevType& D) {
   return D.kind == EK_HEX && m->active != FR_VARIANT_DENSE;
 }
 
+// the viscous flux (9 values a point) is stored at the solution points in
+// place of the gradient (15), which the anti-aliased flux reads
+bool stores_visc(const fr_mesh* m, const DevType& D) {
+  return use_hex(m, D) && m->aa_qdeg == 0;
+}
+
 bool use_tc_grad(const fr_mesh* m, const DevType& D) {
   return D.tc_ok && D.tc_grad_on && m->active == FR_VARIANT_TENSOR;
 }
@@ -1330,7 +1336,9 @@ inline DevType sub_view(const fr_mesh* m, const DevType& D, long long e0, long l
   V.fxs = static_cast<FxCoef*>(sh(D.fxs, 9 * nu * sizeof(FxCoef)));
   V.fxj = static_cast<FxCoef*>(sh(D.fxj, 9 * nu * sizeof(FxCoef)));
   V.fxe = static_cast<int*>(sh(D.fxe, 4 * sizeof(int)));
-  V.grad = sh(D.grad, 15 * nu * w);
+  // [ne][9][nu] where the kernels store the viscous flux: a range's start is
+  // the whole type's, since a stage's phases may run over different ranges
+  V.grad = sh(D.grad, (stores_visc(m, D) ? 9 : 15) * nu * w);
   V.fnv = sh(D.fnv, 3 * nf * w);
   V.fbc = static_cast<int8_t*>(sh(D.fbc, nf));
   V.fbi = static_cast<int32_t*>(sh(D.fbi, nf * sizeof(int32_t)));
