@@ -670,7 +670,8 @@ __global__ void k_exchange_scatter(int n, const int32_t* __restrict__ list,
 // ---------------------------------------------------------------------------
 // Dense kernels (prisms, tetrahedra, and the dense hexahedron variant) are
 // persistent: each CTA copies the type's operators into shared memory once
-// (when they fit) and then loops over groups of EPB elements.
+// (when they fit) and then loops over groups of eb elements (eb NU threads, eb
+// at most EPB; fewer where full groups would leave SMs without any).
 
 // one point's row of 5 / 15 values (16-byte aligned rows)
 template <typename T>
@@ -823,7 +824,7 @@ __device__ __forceinline__ DenseOps<T> stage_dense_ops(const DenseOps<T>& g,
 // the flux points.
 template <typename T, int NU, int NF, int EPB, bool QV>
 __global__ void __launch_bounds__(EPB* NU)
-    k_grad_dense(long long ne, const T* __restrict__ u,
+    k_grad_dense(long long ne, int eb, const T* __restrict__ u,
                  const __grid_constant__ TraceArgs<T> ta, const T* __restrict__ smat,
                  const T* __restrict__ rcpdjac, DenseOps<T> gops,
                  T* __restrict__ grad, ViscArgs<T> va, BCTab<T> bc,
@@ -838,9 +839,9 @@ __global__ void __launch_bounds__(EPB* NU)
   T* us = buf + le * L::kGradElem;             // u at the solution points
   T* ds = us + (L::kRows ? P5 * NU : 5 * NU);  // du at the flux points
   T* gs = ds + (L::kRows ? P5 * NF : 5 * NF);  // physical gradient (15)
-  const long long ngroups = (ne + EPB - 1) / EPB;
+  const long long ngroups = (ne + eb - 1) / eb;
   for (long long grp = blockIdx.x; grp < ngroups; grp += gridDim.x) {
-    const long long e = grp * EPB + le;
+    const long long e = grp * eb + le;
     const bool act = e < ne;
     if (act) {
       T v[5];
@@ -942,7 +943,7 @@ __global__ void __launch_bounds__(EPB* NU)
 // ([ne][3][5][NU], Section 3.2) and is read instead of collocated.
 template <typename T, int NU, int NF, int EPB, bool NS, bool AA = false>
 __global__ void __launch_bounds__(EPB* NU)
-    k_vol_dense(long long ne, const T* __restrict__ u,
+    k_vol_dense(long long ne, int eb, const T* __restrict__ u,
                 const T* __restrict__ grad, const T* __restrict__ fc,
                 const T* __restrict__ smat, const T* __restrict__ rcpdjac,
                 DenseOps<T> gops, Phys<T> ph, StageArgs<T> sa,
@@ -956,9 +957,9 @@ __global__ void __launch_bounds__(EPB* NU)
   const int le = threadIdx.x / NU, z = threadIdx.x % NU;
   T* ft = buf + le * L::kVolElem;  // f~ (component d * 5 + k), then u_next
   T* jm = ft + (L::kRows ? 16 * NU : 15 * NU);  // F^C - n~.f~ at the flux points
-  const long long ngroups = (ne + EPB - 1) / EPB;
+  const long long ngroups = (ne + eb - 1) / eb;
   for (long long grp = blockIdx.x; grp < ngroups; grp += gridDim.x) {
-    const long long e = grp * EPB + le;
+    const long long e = grp * eb + le;
     const bool act = e < ne;
     T uz[5];
     if (act) {

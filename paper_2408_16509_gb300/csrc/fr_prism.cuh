@@ -101,7 +101,7 @@ __device__ __forceinline__ PriOps<T> stage_pri_ops(const PriOps<T>& g, unsigned 
 // its values at the flux points (q form: the viscous normal flux there).
 template <typename T, int NU, int NF, int EPB, bool QV>
 __global__ void __launch_bounds__(EPB* NU)
-    k_grad_pri(long long ne, const T* __restrict__ u,
+    k_grad_pri(long long ne, int eb, const T* __restrict__ u,
                const __grid_constant__ TraceArgs<T> ta,
                const T* __restrict__ smat, const T* __restrict__ rcpdjac, PriOps<T> gops,
                T* __restrict__ grad, ViscArgs<T> va, BCTab<T> bc, Phys<T> ph) {
@@ -116,9 +116,9 @@ __global__ void __launch_bounds__(EPB* NU)
   T* us = buf + le * L::kGradElem;
   T* ds = us + (L::kRows ? L::kP5 * NU : 5 * NU);
   T* gs = ds + (L::kRows ? L::kP5 * NF : 5 * NF);
-  const long long ngroups = (ne + EPB - 1) / EPB;
+  const long long ngroups = (ne + eb - 1) / eb;
   for (long long grp = blockIdx.x; grp < ngroups; grp += gridDim.x) {
-    const long long e = grp * EPB + le;
+    const long long e = grp * eb + le;
     const bool act = e < ne;
     if (act) {
       T v[5];
@@ -219,7 +219,7 @@ __global__ void __launch_bounds__(EPB* NU)
 // the RK epilogue and the next stage's u_f = M0 u_next.
 template <typename T, int NU, int NF, int EPB, bool NS>
 __global__ void __launch_bounds__(EPB* NU)
-    k_vol_pri(long long ne, const T* __restrict__ u, const T* __restrict__ grad,
+    k_vol_pri(long long ne, int eb, const T* __restrict__ u, const T* __restrict__ grad,
               const T* __restrict__ fc, const T* __restrict__ smat,
               const T* __restrict__ rcpdjac, PriOps<T> gops, Phys<T> ph, StageArgs<T> sa) {
   using L = DenseLayout<T, NU, NF>;
@@ -232,9 +232,9 @@ __global__ void __launch_bounds__(EPB* NU)
   const int lz = z / NT, lt = z - lz * NT;
   T* ft = buf + le * L::kVolElem;  // f~ (component d * 5 + k), then u_next
   T* jm = ft + (L::kRows ? 16 * NU : 15 * NU);
-  const long long ngroups = (ne + EPB - 1) / EPB;
+  const long long ngroups = (ne + eb - 1) / eb;
   for (long long grp = blockIdx.x; grp < ngroups; grp += gridDim.x) {
-    const long long e = grp * EPB + le;
+    const long long e = grp * eb + le;
     const bool act = e < ne;
     T uz[5];
     if (act) {
