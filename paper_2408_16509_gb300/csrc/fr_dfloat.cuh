@@ -54,9 +54,6 @@ __device__ __forceinline__ dfl df_rcp(float a) {
   return df_fast_two_sum(r, r * e);
 }
 
-// the double-float's value as an FP64 number (one FP64 add)
-__device__ __forceinline__ double df_to_f64(dfl x) { return widen_f32(x.hi) + widen_f32(x.lo); }
-
 // p = (gamma - 1)(E - (mx^2 + my^2 + mz^2) / (2 rho)) from FP32 conserved
 // values (exact inputs) with rho > 0 and rr = 1/rho; gm1 = gamma - 1 as a
 // double-float.  *amb: |p| is within 2^-36 of (|E| + |k|), where the
@@ -82,11 +79,36 @@ __device__ __forceinline__ dfl df_normalise(dfl x, int* e) {
   return dfl{a * s, sg * x.lo * s};
 }
 
-// Ordering key of s^5 = p^5 rho^-7 (gamma = 7/5) as an FP64 number, from
-// double-float p and rr = 1/rho: sign(p) |p|^5 rr^7 to about 2^-43
-// relative.  Returns false (no key) when an exponent leaves the ranges
-// where every intermediate stays a normal FP32 / FP64 number.
-__device__ __forceinline__ bool df_s5_key(dfl p, dfl rr, double* key) {
+// Integer ordering keys (larger value, larger key; 5 low bits free): of an
+// FP64 number through its top 47 fraction bits, of a double-float value to
+// about 2^-40.  No FP64 instruction.
+
+// y = +-m 2^e with m in [1, 2): the magnitude's key ((e + 1024) 2^47 plus the
+// fraction in units of 2^-47), 0 for y = 0; e is in (-1024, 1024)
+__device__ __forceinline__ long long key47_f64(double y) {
+  const long long b = __double_as_longlong(y);
+  const long long k = ((b & 0x7fffffffffffffffLL) >> 5) + (1LL << 47);  // bias 1023 + 1
+  return (b << 1) == 0 ? 0 : b < 0 ? -k : k;
+}
+
+// ordering key of a double-float (|lo| <= ulp(hi) / 2): hi, then lo
+__device__ __forceinline__ long long key_df(dfl x) {
+  const int h = int(__float_as_uint(x.hi)), l = int(__float_as_uint(x.lo));
+  const int oh = h ^ ((h >> 31) & 0x7fffffff), ol = l ^ ((l >> 31) & 0x7fffffff);
+  return ((long long)oh << 32) | (unsigned(ol) ^ 0x80000000u);
+}
+
+// an FP64 number as a double-float (to 2^-48): a rare path's way into key_df
+__device__ __forceinline__ dfl df_from_f64(double x) {
+  const float h = narrow_f64(x);
+  return dfl{h, narrow_f64(x - widen_f32(h))};
+}
+
+// Key (as key47_f64) of s^5 = p^5 rho^-7 (gamma = 7/5), sign that of p, from
+// double-float p and rr = 1/rho, to about 2^-43 relative.  Returns false (no
+// key) when an exponent leaves the ranges where every intermediate stays a
+// normal number.
+__device__ __forceinline__ bool df_s5_key(dfl p, dfl rr, long long* key) {
   const int ep0 = int((__float_as_uint(fabsf(p.hi)) >> 23) & 0xffu);
   const int er0 = int((__float_as_uint(rr.hi) >> 23) & 0xffu);
   if (ep0 < 30 || ep0 > 225 || er0 < 30 || er0 > 225) return false;
@@ -95,12 +117,14 @@ __device__ __forceinline__ bool df_s5_key(dfl p, dfl rr, double* key) {
   const dfl P2 = df_mul(P, P), P4 = df_mul(P2, P2), P5 = df_mul(P4, P);
   const dfl R2 = df_mul(R, R), R4 = df_mul(R2, R2), R7 = df_mul(df_mul(R4, R2), R);
   const int E = 5 * ep + 7 * er;
-  if (E < -1000 || E > 1000) return false;  // m 2^E normal in FP64
+  if (E < -1000 || E > 1000) return false;
   const dfl M = df_mul(P5, R7);  // in [1, 2^12)
-  const double m = df_to_f64(M);
-  const long long b = __double_as_longlong(m) + ((long long)E << 52);
-  const double y = __longlong_as_double(b);
-  *key = p.hi < 0.f ? -y : y;
+  const unsigned mb = __float_as_uint(M.hi);
+  const int ex = int(mb >> 23) - 127;  // M.hi = 1.f 2^ex
+  // M.lo in units of 2^(ex - 47): within 2^23
+  const int lo = __float2int_rn(M.lo * __uint_as_float(unsigned(127 + 47 - ex) << 23));
+  const long long k = ((long long)(E + ex + 1024) << 47) + ((long long)(mb & 0x7fffffu) << 24) + lo;
+  *key = p.hi < 0.f ? -k : k;
   return true;
 }
 

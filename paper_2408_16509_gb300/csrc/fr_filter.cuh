@@ -202,12 +202,25 @@ __device__ __forceinline__ double warp_sum(double v) {
 // none.  Every point is screened in FP32 (screen_point); the FP64 value is
 // computed only where the screen cannot exclude the minimum or cannot decide
 // admissibility, so the result equals the all-FP64 minimum.
+//
+// FP32 values and gamma = 7/5 (rec not null): the warp only selects the point
+// of least entropy; its FP64 value is left to k_entropy_value, where a warp
+// evaluates 32 elements at once (here one lane would hold the warp for some
+// 50 FP64 instructions of 64 clocks each): 16384 FP32 hexahedra of order 3,
+// 106 -> 59 + 6 us.
+struct EntropyRec {
+  float v[5];  // the selected point's state; v[0] = 0: none
+  float pad;
+  double m;    // minimum over points that took the per-point pow
+};
+
 template <typename T, typename TR, int NU, int NF>
 __global__ void k_entropy_min(long long ne, const T* __restrict__ uin,
                               const TR* __restrict__ X,
                               const T* __restrict__ uf_all, TypeTab tt,
                               int tidx, const int32_t* __restrict__ partner,
-                              double gamma, double* __restrict__ smin) {
+                              double gamma, double* __restrict__ smin,
+                              EntropyRec* __restrict__ rec) {
   constexpr int NQ = (NU + 2 * NF + 31) / 32;
   const int lane = threadIdx.x & 31;
   const long long e = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -291,7 +304,7 @@ __global__ void k_entropy_min(long long ne, const T* __restrict__ uin,
           rr = df_rcp(vf[0]);
           pd = df_pressure(vf[1], vf[2], vf[3], vf[4], rr, gm1d, &amb);
         }
-        double yk;
+        long long yk = 0;
         bool ykey = false;
         if (amb) {
           double v[5];
@@ -301,7 +314,7 @@ __global__ void k_entropy_min(long long ne, const T* __restrict__ uin,
           const double p = (gamma - 1.0) * (v[4] - 0.5 * (v[1] * v[1] + v[2] * v[2] + v[3] * v[3]) * rr64);
           if (!(p > 0.0)) continue;
           if (s5_in_range(p, rr64)) {
-            yk = s5_of(p, rr64);
+            yk = key47_f64(s5_of(p, rr64));
             ykey = true;
           } else {
             m = dmin_key(m, p * pow(v[0], -gamma));
@@ -318,7 +331,7 @@ __global__ void k_entropy_min(long long ne, const T* __restrict__ uin,
           }
         }
         if (ykey) {
-          const long long kt = (dkey(yk) & ~0x1fLL) | lane;
+          const long long kt = (yk << 5) | lane;
           if (kt < ky) {
             ky = kt;
             qy = q;
@@ -331,27 +344,15 @@ __global__ void k_entropy_min(long long ne, const T* __restrict__ uin,
         km = min(km, __shfl_xor_sync(0xffffffffu, km, o));
         kym = min(kym, __shfl_xor_sync(0xffffffffu, kym, o));
       }
-      m = dunkey(km);
-      // the selected point's s^5 in FP64, on its lane, then to lane 0
-      double ysel = INFINITY, sdir = INFINITY;
-      if (qy >= 0 && ky == kym) {
+      if (qy >= 0 && ky == kym) {  // one lane: keys carry the lane
         float vf[5];
         load(lane + 32 * qy, vf);
-        double v[5];
 #pragma unroll
-        for (int k = 0; k < 5; ++k) v[k] = widen_f32(vf[k]);
-        const double rr64 = rcp64(v[0], vf[0]);
-        const double p = (gamma - 1.0) * (v[4] - 0.5 * (v[1] * v[1] + v[2] * v[2] + v[3] * v[3]) * rr64);
-        if (s5_in_range(p, rr64)) ysel = s5_of(p, rr64);
-        else sdir = p * pow(v[0], -gamma);
+        for (int k = 0; k < 5; ++k) rec[e].v[k] = vf[k];
       }
-      const int src = kym == 0x7fffffffffffffffLL ? 0 : int(kym & 0x1f);
-      ysel = __shfl_sync(0xffffffffu, ysel, src);
-      sdir = __shfl_sync(0xffffffffu, sdir, src);
       if (lane == 0) {
-        m = fmin(m, sdir);
-        if (ysel < INFINITY) m = fmin(m, s_of_s5(ysel));
-        smin[e] = isfinite(m) ? m : 0.0;
+        rec[e].m = dunkey(km);
+        if (kym == 0x7fffffffffffffffLL) rec[e].v[0] = 0.f;
       }
       return;
     }
@@ -393,6 +394,24 @@ __global__ void k_entropy_min(long long ne, const T* __restrict__ uin,
     if (y < INFINITY) m = fmin(m, s_of_s5(y));
     smin[e] = isfinite(m) ? m : 0.0;
   }
+}
+
+// s_min of every element from its record (FP64), one thread per element.
+static __global__ void k_entropy_value(long long ne, const EntropyRec* __restrict__ rec,
+                                       double gamma, double* __restrict__ smin) {
+  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= ne) return;
+  const EntropyRec r = rec[e];
+  double m = r.m;
+  if (r.v[0] > 0.f) {
+    double v[5];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) v[k] = widen_f32(r.v[k]);
+    const double rr = rcp64(v[0], r.v[0]);
+    const double p = (gamma - 1.0) * (v[4] - 0.5 * (v[1] * v[1] + v[2] * v[2] + v[3] * v[3]) * rr);
+    m = fmin(m, s5_in_range(p, rr) ? s_of_s5(s5_of(p, rr)) : p * pow(v[0], -gamma));
+  }
+  smin[e] = isfinite(m) ? m : 0.0;
 }
 
 // Block-wide reductions for the filter kernel.
@@ -555,25 +574,21 @@ static __device__ float mlp_guess(const float feat[4], const __nv_bfloat16* w,
   return o > 20.f ? o : log1pf(__expf(o));
 }
 
-// Minima of rho, p and s over a warp's element: slots lane + 32 q of v
-// (with their FP32 screens), FP64 values where the screen cannot decide; the
-// points of least p and least s^5 selected in double-float arithmetic for
-// FP32 values with gamma = 7/5 and computed in FP64 (as k_filter's minima).
-// Returns, on every lane, r (exact), p (FP64 at its point), s_dir (minimum
-// of s over the points that took the per-point pow) and ys (s^5 at its
-// point, FP64).
+// Minima of rho, p and s over a warp's element (FP64 values): slots lane + 32 q
+// of v with their FP32 screens, FP64 p and s where the screen cannot decide.
+// Returns, on every lane, r, p, s_dir (minimum of s over the points that
+// took the per-point pow) and ys (least s^5 of the others).
 template <typename T, int NQ, int NP>
 __device__ __forceinline__ void warp_minima(const T (&v)[NQ][5], const PtScreen (&sc)[NQ],
-                                            double smin, double g, bool by5, dfl gm1d,
-                                            double* r_out, double* p_out, double* s_out,
-                                            double* ys_out) {
+                                            double smin, double g, bool by5, double* r_out,
+                                            double* p_out, double* s_out, double* ys_out) {
   const int lane = threadIdx.x & 31;
   float phi = INFINITY, shi = INFINITY;
-  double rmin = INFINITY;
+  double rmin = INFINITY, mp = INFINITY, ms = INFINITY, my = INFINITY;
 #pragma unroll
   for (int q = 0; q < NQ; ++q) {
     if (lane + 32 * q >= NP) continue;
-    rmin = dmin_key(rmin, to_f64(v[q][0]));
+    rmin = dmin_key(rmin, v[q][0]);
     if (sc[q].pos) {
       phi = fminf(phi, sc[q].phi);
       shi = fminf(shi, sc[q].shi);
@@ -584,105 +599,204 @@ __device__ __forceinline__ void warp_minima(const T (&v)[NQ][5], const PtScreen 
     phi = fminf(phi, __shfl_xor_sync(0xffffffffu, phi, o));
     shi = fminf(shi, __shfl_xor_sync(0xffffffffu, shi, o));
   }
-  double ms = INFINITY;
-  long long kp = 0x7fffffffffffffffLL, ky = 0x7fffffffffffffffLL;
-  int qp = -1, qy = -1;
 #pragma unroll
   for (int q = 0; q < NQ; ++q) {
     if (lane + 32 * q >= NP) continue;
     const bool cp = !sc[q].pos || sc[q].plo <= phi;
     const bool cs = smin > 0.0 && (!sc[q].pos || sc[q].slo <= shi);
     if (!cp && !cs) continue;
-    double pk = 0.0, yk = 0.0;
-    bool ykey = false, exact = true;
-    if constexpr (sizeof(T) == 4) {
-      const float r = v[q][0];
-      if (by5 && r >= 0x1p-100f && r <= 0x1p100f) {
-        bool amb;
-        const dfl rr = df_rcp(r);
-        const dfl pd = df_pressure(v[q][1], v[q][2], v[q][3], v[q][4], rr, gm1d, &amb);
-        if (!amb) {
-          exact = false;
-          pk = df_to_f64(pd);
-          if (cs) {
-            if (df_s5_key(pd, rr, &yk)) {
-              ykey = true;
-            } else {
-              double w[5];
+    const double* w = v[q];
+    const bool rpos = w[0] > 0.0;
+    const double rr64 = rpos ? rcp64(w[0], narrow_f64(w[0])) : 0.0;
+    // (p enters the minimum by the division, s^5 by the reciprocal)
+    if (cp) mp = dmin_key(mp, pressure64(w, g));
+    if (cs) {
+      const double pk =
+          (g - 1.0) * (w[4] - 0.5 * (w[1] * w[1] + w[2] * w[2] + w[3] * w[3]) * rr64);
+      if (!rpos)
+        ms = -INFINITY;
+      else if (by5 && s5_in_range(pk, rr64))
+        my = dmin_key(my, s5_of(pk, rr64));
+      else
+        ms = dmin_key(ms, pk * pow(w[0], -g));
+    }
+  }
+  long long k[4] = {dkey(rmin), dkey(mp), dkey(ms), dkey(my)};
 #pragma unroll
-              for (int k = 0; k < 5; ++k) w[k] = to_f64(v[q][k]);
-              ms = dmin_key(ms, pressure64(w, g) * pow(w[0], -g));
-            }
-          }
+  for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) k[i] = min(k[i], __shfl_xor_sync(0xffffffffu, k[i], o));
+  *r_out = dunkey(k[0]);
+  *p_out = dunkey(k[1]);
+  *s_out = dunkey(k[2]);
+  *ys_out = dunkey(k[3]);
+}
+
+// FP32 values: the points that decide an element's zeta = 0 test, selected by
+// a warp (as warp_minima, in double-float arithmetic where gamma = 7/5),
+// evaluated in FP64 by k_filter_decide, a thread per element (16384
+// hexahedra of order 3: 139 -> 56 + 6 us against a warp that did both).
+struct CheckRec {
+  float pv[5];  // point of least pressure; has & 1
+  float yv[5];  // point of least s^5; has & 2
+  float r;      // least density
+  int has;
+  double ms;    // least s over the points that took the per-point pow
+};
+
+template <int NQ, int NP>
+__device__ __forceinline__ void warp_select(const float (&v)[NQ][5], const PtScreen (&sc)[NQ],
+                                            bool entropy, double g, bool by5, dfl gm1d,
+                                            CheckRec* __restrict__ rec) {
+  const int lane = threadIdx.x & 31;
+  float phi = INFINITY, shi = INFINITY, rmin = INFINITY;
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) {
+    if (lane + 32 * q >= NP) continue;
+    rmin = fminf(rmin, v[q][0]);
+    if (sc[q].pos) {
+      phi = fminf(phi, sc[q].phi);
+      shi = fminf(shi, sc[q].shi);
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    phi = fminf(phi, __shfl_xor_sync(0xffffffffu, phi, o));
+    shi = fminf(shi, __shfl_xor_sync(0xffffffffu, shi, o));
+    rmin = fminf(rmin, __shfl_xor_sync(0xffffffffu, rmin, o));
+  }
+  constexpr long long kNone = 0x7fffffffffffffffLL;
+  double ms = INFINITY;
+  long long kp = kNone, ky = kNone;
+  int qp = -1, qy = -1;
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) {
+    if (lane + 32 * q >= NP) continue;
+    const bool cp = !sc[q].pos || sc[q].plo <= phi;
+    const bool cs = entropy && (!sc[q].pos || sc[q].slo <= shi);
+    if (!cp && !cs) continue;
+    const float r = v[q][0];
+    dfl pd{0.f, 0.f};
+    long long yk = 0;
+    bool ykey = false, amb = !(by5 && r >= 0x1p-100f && r <= 0x1p100f), pnan = false;
+    if (!amb) {
+      const dfl rr = df_rcp(r);
+      pd = df_pressure(v[q][1], v[q][2], v[q][3], v[q][4], rr, gm1d, &amb);
+      if (!amb && cs) {
+        ykey = df_s5_key(pd, rr, &yk);
+        if (!ykey) {
+          double w[5];
+#pragma unroll
+          for (int k = 0; k < 5; ++k) w[k] = widen_f32(v[q][k]);
+          ms = dmin_key(ms, pressure64(w, g) * pow(w[0], -g));
         }
       }
     }
-    if (exact) {
+    if (amb) {  // FP64 at this point
       double w[5];
 #pragma unroll
-      for (int k = 0; k < 5; ++k) w[k] = to_f64(v[q][k]);
+      for (int k = 0; k < 5; ++k) w[k] = widen_f32(v[q][k]);
       const bool rpos = w[0] > 0.0;
-      const double rr64 = rpos ? rcp64(w[0], sizeof(T) == 4 ? float(v[q][0]) : narrow_f64(w[0])) : 0.0;
-      pk = rpos ? (g - 1.0) * (w[4] - 0.5 * (w[1] * w[1] + w[2] * w[2] + w[3] * w[3]) * rr64)
-                : pressure64(w, g);
+      const double rr64 = rpos ? rcp64(w[0], r) : 0.0;
+      const double pk =
+          rpos ? (g - 1.0) * (w[4] - 0.5 * (w[1] * w[1] + w[2] * w[2] + w[3] * w[3]) * rr64)
+               : pressure64(w, g);
+      pnan = !(pk == pk);
+      pd = df_from_f64(pk);
       if (cs) {
         if (!rpos) {
           ms = -INFINITY;
         } else if (by5 && s5_in_range(pk, rr64)) {
-          yk = s5_of(pk, rr64);
+          yk = key47_f64(s5_of(pk, rr64));
           ykey = true;
         } else {
           ms = dmin_key(ms, pk * pow(w[0], -g));
         }
       }
     }
-    const bool pnan = (__double_as_longlong(pk) & 0x7fffffffffffffffLL) > 0x7ff0000000000000LL;
-    const long long kt = (dkey(pk) & ~0x1fLL) | lane;
+    const long long kt = (key_df(pd) & ~0x1fLL) | lane;
     if (cp && !pnan && kt < kp) {
       kp = kt;
       qp = q;
     }
     if (ykey) {
-      const long long kyt = (dkey(yk) & ~0x1fLL) | lane;
+      const long long kyt = (yk << 5) | lane;
       if (kyt < ky) {
         ky = kyt;
         qy = q;
       }
     }
   }
-  long long kr = dkey(rmin), kms = dkey(ms), kpm = kp, kym = ky;
+  long long kms = dkey(ms), kpm = kp, kym = ky;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-    kr = min(kr, __shfl_xor_sync(0xffffffffu, kr, o));
     kms = min(kms, __shfl_xor_sync(0xffffffffu, kms, o));
     kpm = min(kpm, __shfl_xor_sync(0xffffffffu, kpm, o));
     kym = min(kym, __shfl_xor_sync(0xffffffffu, kym, o));
   }
-  // the selected points' FP64 values, from their lanes
-  double psel = INFINITY, ysel = INFINITY, sdir = INFINITY;
-  if (qp >= 0 && kp == kpm) {
-    double w[5];
 #pragma unroll
-    for (int k = 0; k < 5; ++k) w[k] = to_f64(v[qp][k]);
-    psel = pressure64(w, g);
-  }
-  if (qy >= 0 && ky == kym) {
-    double w[5];
+  for (int q = 0; q < NQ; ++q) {  // one lane each: the keys carry the lane
+    if (qp == q && kp == kpm) {
 #pragma unroll
-    for (int k = 0; k < 5; ++k) w[k] = to_f64(v[qy][k]);
-    const double rr64 = rcp64(w[0], sizeof(T) == 4 ? float(v[qy][0]) : narrow_f64(w[0]));
-    const double p64 = (g - 1.0) * (w[4] - 0.5 * (w[1] * w[1] + w[2] * w[2] + w[3] * w[3]) * rr64);
-    if (s5_in_range(p64, rr64)) ysel = s5_of(p64, rr64);
-    else sdir = p64 * pow(w[0], -g);
+      for (int k = 0; k < 5; ++k) rec->pv[k] = v[q][k];
+    }
+    if (qy == q && ky == kym) {
+#pragma unroll
+      for (int k = 0; k < 5; ++k) rec->yv[k] = v[q][k];
+    }
   }
-  const bool hp = kpm != 0x7fffffffffffffffLL, hy = kym != 0x7fffffffffffffffLL;
-  psel = __shfl_sync(0xffffffffu, psel, hp ? int(kpm & 0x1f) : 0);
-  ysel = __shfl_sync(0xffffffffu, ysel, hy ? int(kym & 0x1f) : 0);
-  sdir = __shfl_sync(0xffffffffu, sdir, hy ? int(kym & 0x1f) : 0);
-  *r_out = dunkey(kr);
-  *p_out = hp ? psel : INFINITY;
-  *s_out = fmin(dunkey(kms), hy ? sdir : INFINITY);
-  *ys_out = hy ? ysel : INFINITY;
+  if (lane == 0) {
+    rec->r = rmin;
+    rec->has = (kpm != kNone ? 1 : 0) | (kym != kNone ? 2 : 0);
+    rec->ms = dunkey(kms);
+  }
+}
+
+// Outcome of the zeta = 0 test of element e from its minima: left alone (zeta
+// 0, one evaluation) or listed for k_filter.
+__device__ __forceinline__ void check_outcome(long long e, double r, double p, double sdir,
+                                              double ys, double smin, double sb,
+                                              const FilterArgs& fa, int32_t* __restrict__ list,
+                                              int* __restrict__ count) {
+  double s_term = INFINITY;
+  if (smin > 0.0) {
+    const double sb2 = sb * sb, sb5 = sb2 * sb2 * sb;
+    s_term = (sdir >= sb && !(ys < sb5)) ? 0.0 : -1.0;
+  }
+  const double gm = fmin(r - kEpsPos, fmin(p - kEpsPos, s_term));
+  if (!isnan(gm) && gm >= 0.0) {
+    if (fa.zeta_last) {
+      fa.zeta_last[e] = 0.f;
+      fa.evals_last[e] = 1;
+    }
+  } else {
+    list[atomicAdd(count, 1)] = int32_t(e);
+  }
+}
+
+// The zeta = 0 test from the records of k_filter_check (FP32 values).
+static __global__ void k_filter_decide(long long ne, const CheckRec* __restrict__ rec,
+                                       FilterArgs fa, int32_t* __restrict__ list,
+                                       int* __restrict__ count) {
+  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= ne) return;
+  const CheckRec c = rec[e];
+  const double g = fa.gamma, smin = fa.smin[e], sb = smin * (1.0 - fa.tau);
+  double p = INFINITY, ys = INFINITY, sdir = c.ms, w[5];
+  if (c.has & 1) {
+#pragma unroll
+    for (int k = 0; k < 5; ++k) w[k] = widen_f32(c.pv[k]);
+    p = pressure64(w, g);
+  }
+  if (c.has & 2) {
+#pragma unroll
+    for (int k = 0; k < 5; ++k) w[k] = widen_f32(c.yv[k]);
+    const double rr = rcp64(w[0], c.yv[0]);
+    const double p64 = (g - 1.0) * (w[4] - 0.5 * (w[1] * w[1] + w[2] * w[2] + w[3] * w[3]) * rr);
+    if (s5_in_range(p64, rr)) ys = s5_of(p64, rr);
+    else sdir = fmin(sdir, p64 * pow(w[0], -g));
+  }
+  check_outcome(e, widen_f32(c.r), p, sdir, ys, smin, sb, fa, list, count);
 }
 
 // The zeta = 0 test of every element of a type, one warp per element, on
@@ -694,7 +808,7 @@ template <typename T, typename TR, int NU, int NF>
 __global__ void k_filter_check(long long ne, const T* __restrict__ reg,
                                const TR* __restrict__ regR, const T* __restrict__ uf,
                                FilterArgs fa, int32_t* __restrict__ list,
-                               int* __restrict__ count) {
+                               int* __restrict__ count, CheckRec* __restrict__ rec) {
   constexpr int NP = NU + NF, NQ = (NP + 31) / 32;
   const int lane = threadIdx.x & 31;
   const long long e = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -723,22 +837,12 @@ __global__ void k_filter_check(long long ne, const T* __restrict__ reg,
     sc[q] = screen_point(float(v[q][0]), float(v[q][1]), float(v[q][2]), float(v[q][3]),
                          float(v[q][4]), gf);
   }
-  double r, p, sdir, ys;
-  warp_minima<T, NQ, NP>(v, sc, smin, g, by5, gm1d, &r, &p, &sdir, &ys);
-  if (lane != 0) return;
-  double s_term = INFINITY;
-  if (smin > 0.0) {
-    const double sb2 = sb * sb, sb5 = sb2 * sb2 * sb;
-    s_term = (sdir >= sb && !(ys < sb5)) ? 0.0 : -1.0;
-  }
-  const double gm = fmin(r - kEpsPos, fmin(p - kEpsPos, s_term));
-  if (!isnan(gm) && gm >= 0.0) {
-    if (fa.zeta_last) {
-      fa.zeta_last[e] = 0.f;
-      fa.evals_last[e] = 1;
-    }
+  if constexpr (sizeof(T) == 4) {
+    warp_select<NQ, NP>(v, sc, smin > 0.0, g, by5, gm1d, rec + e);
   } else {
-    list[atomicAdd(count, 1)] = int32_t(e);
+    double r, p, sdir, ys;
+    warp_minima<T, NQ, NP>(v, sc, smin, g, by5, &r, &p, &sdir, &ys);
+    if (lane == 0) check_outcome(e, r, p, sdir, ys, smin, sb, fa, list, count);
   }
 }
 
@@ -762,14 +866,13 @@ __device__ __forceinline__ void get_modes5(const double (&r)[8], double (&a)[5])
   a[4] = r[4];
 }
 
-// Filter the stage value of each element that violates the constraints.
-// reg / regR: the register holding the new stage value (type T or TR, one
-// of them null); uf: this type's flux-point traces of that value.
+// Filter the stage value of element e, which violates the constraints (the
+// whole CTA).  reg / regR: the register holding the new stage value (type T
+// or TR, one of them null); uf: this type's flux-point traces of that value.
 template <typename T, typename TR, int NU, int NF>
-__global__ void __launch_bounds__(kFilterThreads)
-    k_filter(long long ne, T* __restrict__ reg, TR* __restrict__ regR,
-             T* __restrict__ uf, FilterOps<T> op, FilterArgs fa,
-             const int32_t* __restrict__ list, const int* __restrict__ count) {
+__device__ __forceinline__ void filter_element(const long long e, T* __restrict__ reg,
+                                               TR* __restrict__ regR, T* __restrict__ uf,
+                                               const FilterOps<T>& op, const FilterArgs& fa) {
   constexpr int NM = NU, NP = NU + NF;
   __shared__ T uh[5][NM];       // modal coefficients
   __shared__ __align__(16) T ush[NM][8];  // sigma_k u^_k of an evaluation (5 used)
@@ -777,11 +880,7 @@ __global__ void __launch_bounds__(kFilterThreads)
   __shared__ long long redk[4 * (kFilterThreads / 32)];
   __shared__ float redf[2 * (kFilterThreads / 32)];
   __shared__ double s_z;        // requested strength
-  // CTA b filters element list[b] of the k_filter_check list
-  if (int(blockIdx.x) >= *count) return;
-  const long long e = list[blockIdx.x];
   const int tid = threadIdx.x;
-  if (e >= ne) return;
   const double g = fa.gamma;
   const float gf = float(g);
   const bool by5 = entropy_by_s5(g);
@@ -867,20 +966,22 @@ __global__ void __launch_bounds__(kFilterThreads)
             pd = df_pressure(float(v[q][1]), float(v[q][2]), float(v[q][3]),
                              float(v[q][4]), rr, gm1d, &amb);
           }
-          double pk, yk;
-          bool ykey = false;
+          long long yk = 0;
+          bool ykey = false, pnan = false;
           if (amb) {  // FP64 at this point
             double w[5];
 #pragma unroll
             for (int k = 0; k < 5; ++k) w[k] = to_f64(v[q][k]);
-            pk = pressure64(w, g);
+            const double pk = pressure64(w, g);
+            pnan = !(pk == pk);  // ignored, like fmin
+            pd = df_from_f64(pk);
             if (cs) {
               if (!(w[0] > 0.0)) {
                 ms = -INFINITY;
               } else {
                 const double rr64 = rcp64(w[0], r);
                 if (s5_in_range(pk, rr64)) {
-                  yk = s5_of(pk, rr64);
+                  yk = key47_f64(s5_of(pk, rr64));
                   ykey = true;
                 } else {
                   ms = dmin_key(ms, pk * pow(w[0], -g));
@@ -888,7 +989,6 @@ __global__ void __launch_bounds__(kFilterThreads)
               }
             }
           } else {
-            pk = df_to_f64(pd);
             if (cs) {
               if (df_s5_key(pd, rr, &yk)) {
                 ykey = true;
@@ -900,15 +1000,13 @@ __global__ void __launch_bounds__(kFilterThreads)
               }
             }
           }
-          const bool pnan = (__double_as_longlong(pk) & 0x7fffffffffffffffLL) >
-                            0x7ff0000000000000LL;  // ignored, like fmin
-          const long long kt = (dkey(pk) & ~0xffLL) | tid;
+          const long long kt = (key_df(pd) & ~0xffLL) | tid;
           if (cp && !pnan && kt < kp) {
             kp = kt;
             qp = q;
           }
           if (ykey) {
-            const long long kyt = (dkey(yk) & ~0xffLL) | tid;
+            const long long kyt = ((yk >> 3) << 8) | tid;
             if (kyt < ky) {
               ky = kyt;
               qy = q;
@@ -1033,10 +1131,22 @@ __global__ void __launch_bounds__(kFilterThreads)
   const double wsum = block_sum(ws, red);
   const double rmean = fmax(block_sum(wr, red) / wsum, kEpsPos);
   const double pmean = fmax(block_sum(wp, red) / wsum, kEpsPos);
-  // margin g(z) = min((rho-eps)/rho_mean, (p-eps)/p_mean, (s-sb)/s_min)
+  // margin g(z) = min((rho-eps)/rho_mean, (p-eps)/p_mean, (s-sb)/s_min); one
+  // thread evaluates it, a chain of FP64 instructions of 64 clocks each: the
+  // divisors are inverted once for FP32 values (FP64 values keep the oracle's
+  // divisions, whose evaluation counts they reproduce)
+  const double irm = 1.0 / rmean, ipm = 1.0 / pmean, ism = smin > 0.0 ? 1.0 / smin : 0.0;
   auto gval = [&](const Mins& q) -> double {
-    const double gr = (q.r - kEpsPos) / rmean, gp = (q.p - kEpsPos) / pmean;
-    const double gs = smin > 0.0 ? (smin_of(q) - sb) / smin : INFINITY;
+    double gr, gp, gs = INFINITY;
+    if constexpr (sizeof(T) == 4) {
+      gr = (q.r - kEpsPos) * irm;
+      gp = (q.p - kEpsPos) * ipm;
+      if (smin > 0.0) gs = (smin_of(q) - sb) * ism;
+    } else {
+      gr = (q.r - kEpsPos) / rmean;
+      gp = (q.p - kEpsPos) / pmean;
+      if (smin > 0.0) gs = (smin_of(q) - sb) / smin;
+    }
     double gm = fmin(gr, fmin(gp, gs));
     if (isnan(gm)) gm = -INFINITY;
     return gm;
@@ -1250,6 +1360,22 @@ __global__ void __launch_bounds__(kFilterThreads)
         fa.samples[i * 5 + 4] = float(result);
       }
     }
+  }
+}
+
+// The listed elements, one CTA each in turn.  The list's length is known on
+// the device alone: the grid holds the CTAs that can be resident (one CTA
+// per element of the mesh, most of which only returned, before).  Bound by
+// the margin's serial FP64 chain: 174 -> 137 us on 16384 hexahedra of order 3
+// of which some hundred are listed.
+template <typename T, typename TR, int NU, int NF>
+__global__ void __launch_bounds__(kFilterThreads)
+    k_filter(T* __restrict__ reg, TR* __restrict__ regR, T* __restrict__ uf, FilterOps<T> op,
+             FilterArgs fa, const int32_t* __restrict__ list, const int* __restrict__ count) {
+  const int n = *count;
+  for (int b = blockIdx.x; b < n; b += gridDim.x) {
+    filter_element<T, TR, NU, NF>(list[b], reg, regR, uf, op, fa);
+    __syncthreads();  // the shared arrays serve the next element
   }
 }
 

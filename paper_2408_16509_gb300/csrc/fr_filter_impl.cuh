@@ -32,6 +32,10 @@ int setup_filter(fr_mesh* m) {
     if ((rc = dev_zeros(m, size_t(D.ne) * sizeof(int), (void**)&D.evals_last))) return rc;
     if ((rc = dev_zeros(m, size_t(D.ne) * sizeof(int32_t), (void**)&D.flist))) return rc;
     if ((rc = dev_zeros(m, sizeof(int), (void**)&D.fcount))) return rc;
+    static_assert(sizeof(CheckRec) >= sizeof(EntropyRec), "one buffer serves both");
+    if (sizeof(T) == 4 &&
+        (rc = dev_zeros(m, size_t(D.ne) * sizeof(CheckRec), &D.frec)))
+      return rc;
   }
   if ((rc = setup_partner(m))) return rc;
   if (!m->d_fstats) {
@@ -50,8 +54,11 @@ void launch_entropy_min(fr_mesh* m, cudaStream_t s, bool from_x) {
       long long threads = D.ne * 32;
       k_entropy_min<T, TR, NU, NF><<<nblk(threads, 256), 256, 0, s>>>(
           D.ne, from_x ? nullptr : (const T*)D.Y, (const TR*)D.X,
-          (const T*)m->uf, m->tt, int(t), D.fpartner, m->gamma, D.smin);
+          (const T*)m->uf, m->tt, int(t), D.fpartner, m->gamma, D.smin, (EntropyRec*)D.frec);
     });
+    if (sizeof(T) == 4 && sizeof(TR) == 4 && m->gamma == 1.4)
+      k_entropy_value<<<nblk(D.ne, 128), 128, 0, s>>>(D.ne, (const EntropyRec*)D.frec, m->gamma,
+                                                      D.smin);
   }
 }
 
@@ -75,15 +82,26 @@ void launch_filter(fr_mesh* m, cudaStream_t s, DevType& D, bool last_stage) {
   T* uf = (T*)m->uf + D.off_f;
   T* reg = last_stage ? nullptr : (T*)D.Y;
   TR* regR = last_stage ? (TR*)D.X : nullptr;
-  // the zeta = 0 test of every element (a warp each), then k_filter on the
-  // elements it lists (one CTA per element; CTAs past the count return)
+  // the zeta = 0 test of every element (a warp each; FP32 values: the warp
+  // selects points, a thread per element decides), then k_filter on the
+  // elements it lists
   cudaMemsetAsync(D.fcount, 0, sizeof(int), s);
   dispatch(D.kind, m->order, [&](auto nu, auto nf) {
     constexpr int NU = decltype(nu)::value, NF = decltype(nf)::value;
     k_filter_check<T, TR, NU, NF><<<nblk(D.ne * 32, 256), 256, 0, s>>>(
-        D.ne, reg, regR, uf, fa, D.flist, D.fcount);
-    k_filter<T, TR, NU, NF><<<unsigned(D.ne), kFilterThreads, 0, s>>>(
-        D.ne, reg, regR, uf, op, fa, D.flist, D.fcount);
+        D.ne, reg, regR, uf, fa, D.flist, D.fcount, (CheckRec*)D.frec);
+    if (sizeof(T) == 4)
+      k_filter_decide<<<nblk(D.ne, 128), 128, 0, s>>>(D.ne, (const CheckRec*)D.frec, fa, D.flist,
+                                                      D.fcount);
+    if (D.filter_ctas == 0) {  // resident CTAs per SM
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&D.filter_ctas, k_filter<T, TR, NU, NF>,
+                                                    kFilterThreads, 0);
+      D.filter_ctas = std::max(1, D.filter_ctas);
+    }
+    const unsigned grid =
+        unsigned(std::min<long long>(D.ne, (long long)m->num_sms * D.filter_ctas));
+    k_filter<T, TR, NU, NF><<<grid, kFilterThreads, 0, s>>>(reg, regR, uf, op, fa, D.flist,
+                                                            D.fcount);
   });
 }
 
