@@ -73,15 +73,25 @@ constexpr int dense_epb() {
 }
 
 template <typename T, int NU, int NF>
-constexpr size_t dense_grad_smem() {
+constexpr size_t dense_grad_smem(int eb = dense_epb<NU>()) {
   return (size_t(DenseLayout<T, NU, NF>::kStagedCount) +
-          size_t(dense_epb<NU>()) * size_t(DenseLayout<T, NU, NF>::kGradElem)) * sizeof(T);
+          size_t(eb) * size_t(DenseLayout<T, NU, NF>::kGradElem)) * sizeof(T);
 }
 
 template <typename T, int NU, int NF>
-constexpr size_t dense_vol_smem() {
+constexpr size_t dense_vol_smem(int eb = dense_epb<NU>()) {
   return (size_t(DenseLayout<T, NU, NF>::kStagedCount) +
-          size_t(dense_epb<NU>()) * size_t(DenseLayout<T, NU, NF>::kVolElem)) * sizeof(T);
+          size_t(eb) * size_t(DenseLayout<T, NU, NF>::kVolElem)) * sizeof(T);
+}
+
+// Elements per CTA of those kernels for ne elements: dense_epb, or, when
+// that leaves SMs without a CTA, one group per SM (a warp at least).  756 FP64
+// tetrahedra of order 2 filled 31 CTAs of 25 elements: gradient kernel 63 ->
+// 39 us on 152 CTAs of 5.
+template <int NU>
+inline int dense_eb(long long ne, int num_sms) {
+  const long long per = (ne + num_sms - 1) / num_sms;
+  return int(std::min<long long>(dense_epb<NU>(), std::max<long long>(per, (31 + NU) / NU)));
 }
 
 struct DevType {
@@ -118,6 +128,8 @@ struct DevType {
   void* fW = nullptr;
   int32_t* flist = nullptr;  // [ne] elements that fail the zeta = 0 test
   int* fcount = nullptr;     // their number
+  void* frec = nullptr;      // [ne] EntropyRec / CheckRec (FP32 values)
+  int filter_ctas = 0;       // resident k_filter CTAs per SM (0: not asked yet)
   double* smin = nullptr;
   float* zeta_last = nullptr;
   int* evals_last = nullptr;
@@ -952,15 +964,15 @@ bool use_pri(const fr_mesh* m, const DevType& D) {
 }
 
 template <typename T, int NU, int NF>
-size_t pri_grad_smem(const DevType& D) {
+size_t pri_grad_smem(const DevType& D, int eb = dense_epb<NU>()) {
   return size_t(PriLayout<T, NU, NF>::bytes(D.pri_nm, D.pri_nl)) +
-         size_t(dense_epb<NU>()) * size_t(DenseLayout<T, NU, NF>::kGradElem) * sizeof(T);
+         size_t(eb) * size_t(DenseLayout<T, NU, NF>::kGradElem) * sizeof(T);
 }
 
 template <typename T, int NU, int NF>
-size_t pri_vol_smem(const DevType& D) {
+size_t pri_vol_smem(const DevType& D, int eb = dense_epb<NU>()) {
   return size_t(PriLayout<T, NU, NF>::bytes(D.pri_nm, D.pri_nl)) +
-         size_t(dense_epb<NU>()) * size_t(DenseLayout<T, NU, NF>::kVolElem) * sizeof(T);
+         size_t(eb) * size_t(DenseLayout<T, NU, NF>::kVolElem) * sizeof(T);
 }
 
 // Anti-aliased transformed flux of one element type (Section 3.2) into D.tf;
@@ -1493,12 +1505,13 @@ void launch_stage(fr_mesh* m, cudaStream_t s, int mode, int stage,
           constexpr int NU = decltype(nu)::value, NF = decltype(nf)::value;
           if constexpr (pri_order(NU, NF) > 0) {
             constexpr int E = dense_epb<NU>();
+            const int eb = dense_eb<NU>(D.ne, m->num_sms);
             const unsigned grid = unsigned(std::min<long long>(
-                (D.ne + E - 1) / E,
+                (D.ne + eb - 1) / eb,
                 (long long)m->num_sms * (D.tile_grad > 0 ? D.tile_grad : D.pri_grad_ctas)));
             k_grad_pri<T, NU, NF, E, sizeof(T) == 4>
-                <<<grid, E * NU, pri_grad_smem<T, NU, NF>(D), s>>>(
-                    D.ne, from_x ? (const T*)D.X : (const T*)D.Y, ta, (const T*)D.smat,
+                <<<grid, eb * NU, pri_grad_smem<T, NU, NF>(D, eb), s>>>(
+                    D.ne, eb, from_x ? (const T*)D.X : (const T*)D.Y, ta, (const T*)D.smat,
                     (const T*)D.rcpdjac, pri_ops_of<T>(m, D), (T*)D.grad, va, bc, ph);
           }
         });
@@ -1506,12 +1519,13 @@ void launch_stage(fr_mesh* m, cudaStream_t s, int mode, int stage,
         dispatch(D.kind, m->order, [&](auto nu, auto nf) {
           constexpr int NU = decltype(nu)::value, NF = decltype(nf)::value;
           constexpr int E = dense_epb<NU>();
-          const size_t sm = dense_grad_smem<T, NU, NF>();
+          const int eb = dense_eb<NU>(D.ne, m->num_sms);
+          const size_t sm = dense_grad_smem<T, NU, NF>(eb);
           const unsigned grid = unsigned(std::min<long long>(
-              (D.ne + E - 1) / E,
+              (D.ne + eb - 1) / eb,
               (long long)m->num_sms * (D.tile_grad > 0 ? D.tile_grad : D.grad_ctas)));
-          k_grad_dense<T, NU, NF, E, sizeof(T) == 4><<<grid, E * NU, sm, s>>>(
-              D.ne, from_x ? (const T*)D.X : (const T*)D.Y, ta,
+          k_grad_dense<T, NU, NF, E, sizeof(T) == 4><<<grid, eb * NU, sm, s>>>(
+              D.ne, eb, from_x ? (const T*)D.X : (const T*)D.Y, ta,
               (const T*)D.smat, (const T*)D.rcpdjac, stage_ops_of<T>(m, D), (T*)D.grad,
               va, bc, ph);
         });
@@ -1637,17 +1651,18 @@ void launch_stage(fr_mesh* m, cudaStream_t s, int mode, int stage,
           constexpr int NU = decltype(nu)::value, NF = decltype(nf)::value;
           if constexpr (pri_order(NU, NF) > 0) {
             constexpr int E = dense_epb<NU>();
+            const int eb = dense_eb<NU>(D.ne, m->num_sms);
             const unsigned grid = unsigned(std::min<long long>(
-                (D.ne + E - 1) / E,
+                (D.ne + eb - 1) / eb,
                 (long long)m->num_sms * (D.tile_vol > 0 ? D.tile_vol : D.pri_vol_ctas)));
-            const size_t sm = pri_vol_smem<T, NU, NF>(D);
+            const size_t sm = pri_vol_smem<T, NU, NF>(D, eb);
             if (ns)
-              k_vol_pri<T, NU, NF, E, true><<<grid, E * NU, sm, s>>>(
-                  D.ne, uin, (const T*)D.grad, fc, (const T*)D.smat, (const T*)D.rcpdjac,
+              k_vol_pri<T, NU, NF, E, true><<<grid, eb * NU, sm, s>>>(
+                  D.ne, eb, uin, (const T*)D.grad, fc, (const T*)D.smat, (const T*)D.rcpdjac,
                   pri_ops_of<T>(m, D), ph, sa);
             else
-              k_vol_pri<T, NU, NF, E, false><<<grid, E * NU, sm, s>>>(
-                  D.ne, uin, nullptr, fc, (const T*)D.smat, (const T*)D.rcpdjac,
+              k_vol_pri<T, NU, NF, E, false><<<grid, eb * NU, sm, s>>>(
+                  D.ne, eb, uin, nullptr, fc, (const T*)D.smat, (const T*)D.rcpdjac,
                   pri_ops_of<T>(m, D), ph, sa);
           }
         });
@@ -1655,21 +1670,22 @@ void launch_stage(fr_mesh* m, cudaStream_t s, int mode, int stage,
       dispatch(D.kind, m->order, [&](auto nu, auto nf) {
         constexpr int NU = decltype(nu)::value, NF = decltype(nf)::value;
         constexpr int E = dense_epb<NU>();
-        const size_t sm = dense_vol_smem<T, NU, NF>();
+        const int eb = dense_eb<NU>(D.ne, m->num_sms);
+        const size_t sm = dense_vol_smem<T, NU, NF>(eb);
         const unsigned grid = unsigned(std::min<long long>(
-            (D.ne + E - 1) / E,
+            (D.ne + eb - 1) / eb,
             (long long)m->num_sms * (D.tile_vol > 0 ? D.tile_vol : D.vol_ctas)));
         if (aa)
-          k_vol_dense<T, NU, NF, E, false, true><<<grid, E * NU, sm, s>>>(
-              D.ne, uin, nullptr, fc, nullptr, (const T*)D.rcpdjac,
+          k_vol_dense<T, NU, NF, E, false, true><<<grid, eb * NU, sm, s>>>(
+              D.ne, eb, uin, nullptr, fc, nullptr, (const T*)D.rcpdjac,
               stage_ops_of<T>(m, D), ph, sa, (const T*)D.tf);
         else if (ns)
-          k_vol_dense<T, NU, NF, E, true><<<grid, E * NU, sm, s>>>(
-              D.ne, uin, (const T*)D.grad, fc, (const T*)D.smat,
+          k_vol_dense<T, NU, NF, E, true><<<grid, eb * NU, sm, s>>>(
+              D.ne, eb, uin, (const T*)D.grad, fc, (const T*)D.smat,
               (const T*)D.rcpdjac, stage_ops_of<T>(m, D), ph, sa);
         else
-          k_vol_dense<T, NU, NF, E, false><<<grid, E * NU, sm, s>>>(
-              D.ne, uin, nullptr, fc, (const T*)D.smat, (const T*)D.rcpdjac,
+          k_vol_dense<T, NU, NF, E, false><<<grid, eb * NU, sm, s>>>(
+              D.ne, eb, uin, nullptr, fc, (const T*)D.smat, (const T*)D.rcpdjac,
               stage_ops_of<T>(m, D), ph, sa);
       });
     }
