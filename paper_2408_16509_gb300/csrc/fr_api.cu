@@ -933,8 +933,15 @@ int fr_set_schedule(fr_mesh* m, const fr_schedule_t* in) {
     const DevType& D = m->types[t];
     const bool hexk = D.kind == EK_HEX && m->active != FR_VARIANT_DENSE;
     const bool prik = use_pri(m, D);
-    const int mg = hexk ? hex_tile_max(m->order) : prik ? D.pri_grad_ctas : D.grad_ctas;
-    const int mv = hexk ? hex_tile_max(m->order) : prik ? D.pri_vol_ctas : D.vol_ctas;
+    int mg = hexk ? hex_tile_max(m->order) : prik ? D.pri_grad_ctas : D.grad_ctas;
+    int mv = hexk ? hex_tile_max(m->order) : prik ? D.pri_vol_ctas : D.vol_ctas;
+    if (use_simplex(m, D)) {
+      // more CTAs per SM than can be resident run as the most that can: a
+      // schedule saved with the kernels of one thread per point (at most 8
+      // CTAs of 256 threads) stays valid
+      mg = std::max(8, D.sx_grad_ctas);
+      mv = std::max(8, D.sx_vol_ctas);
+    }
     if (in->tile_grad[k] < 0 || in->tile_grad[k] > mg || in->tile_vol[k] < 0 ||
         in->tile_vol[k] > mv)
       return fail(FR_EINVAL, "tile out of range for this kernel");

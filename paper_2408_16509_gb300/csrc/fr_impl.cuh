@@ -28,6 +28,7 @@
 #include "fr_hexline.cuh"
 #include "fr_kernels.cuh"
 #include "fr_prism.cuh"
+#include "fr_simplex.cuh"
 #include "fr_err.hpp"
 #include "fr_mesh.hpp"
 
@@ -140,6 +141,11 @@ struct DevType {
   int pri_nm = 0, pri_nl = 0;
   void* pri_img = nullptr;
   int pri_grad_ctas = 1, pri_vol_ctas = 1;
+  // tetrahedra and prisms, FP32 values: operators of fr_simplex.cuh for the
+  // gradient and the volume kernel
+  bool sx_ok = false;
+  SimplexOps sx_grad{}, sx_vol{};
+  int sx_grad_ctas = 1, sx_vol_ctas = 1;
   // tetrahedra: M0 by its nonzeros (every flux point is a solution point)
   int32_t* m0c = nullptr;
   void* m0v = nullptr;
@@ -414,6 +420,120 @@ inline bool build_prism_ops(const RefElement& R, std::vector<double>& tv,
   for (int i = 0; i < 3 * NF; ++i) nr[i] = R.fnorm[i];
   *nm_out = nm;
   *nl_out = nl;
+  return true;
+}
+
+// Operators of the blocked FP32 kernels (fr_simplex.cuh), output points in
+// groups of zb: the image of SimplexOps and the vectors kept as arguments.
+// Tetrahedra need one reference normal per face; prisms also the structure of
+// build_prism_ops, and a LIFT whose triangle columns act along a line and
+// whose quadrilateral columns act within a level, 3 (p + 1) a level.  Entries
+// below 1e-12 of an operator's largest are structural zeros.  Returns false
+// (the other kernels stay) when any of it does not hold.
+template <int NU, int NF>
+bool build_simplex_ops(const RefElement& R, int zb, std::vector<uint32_t>& img, SimplexOps& o) {
+  using G = SimplexGeom<NU, NF>;
+  constexpr bool pri = G::P > 0;
+  if (R.nupts != NU || R.nfpts != NF || R.kind != (pri ? EK_PRI : EK_TET)) return false;
+  auto amax = [](const std::vector<double>& v) {
+    double a = 0.0;
+    for (double x : v) a = std::max(a, std::fabs(x));
+    return a;
+  };
+  const double tm = 1e-12 * amax(R.M0), tl = 1e-12 * amax(R.LIFT);
+  auto lift = [&](int z, int f) { return R.LIFT[size_t(z) * NF + f]; };
+  auto face = [&](int f) {
+    return !pri ? f / G::NT : f < 2 * G::NT ? f / G::NT : 2 + (f - 2 * G::NT) / (G::NL * G::NL);
+  };
+  std::vector<int> first(kSimplexMaxFaces, -1);
+  for (int f = 0; f < NF; ++f) {
+    const int fa = face(f);
+    if (first[fa] < 0) first[fa] = f;
+    for (int d = 0; d < 3; ++d) {
+      const double n = R.fnorm[size_t(f) * 3 + d];
+      if (std::fabs(n - R.fnorm[size_t(first[fa]) * 3 + d]) > 1e-12) return false;
+      if (pri && (fa < 2) != (d == 2) && std::fabs(n) > 1e-12) return false;
+      o.nface[fa][d] = float(n);
+    }
+  }
+  int nm = 0;
+  for (int f = 0; f < NF; ++f) {
+    int c = 0;
+    for (int q = 0; q < NU; ++q) c += std::fabs(R.M0[size_t(f) * NU + q]) > tm;
+    nm = std::max(nm, c);
+  }
+  if (nm < 1 || nm > kPriMaxM0 || (!pri && 4 * nm > NU)) return false;
+  o.nm = nm;
+  img.assign(size_t(G::words(zb, nm)), 0u);
+  auto put = [&](size_t i, double v) {
+    const float x = float(v);
+    std::memcpy(&img[i], &x, 4);
+  };
+  const int ng = G::ng(zb), gp = G::gp(zb);
+  auto col = [&](int z) { return size_t(z / zb) * gp + z % zb; };  // within ng groups
+  const size_t w = size_t(ng) * gp, m0v = size_t(G::ops(zb)), m0c = m0v + G::m0(nm);
+  if constexpr (!pri) {
+    for (int q = 0; q < NU; ++q)
+      for (int d = 0; d < 3; ++d)
+        for (int z = 0; z < NU; ++z)
+          put((size_t(q) * 3 + d) * w + col(z), R.D[(size_t(d) * NU + z) * NU + q]);
+    for (int f = 0; f < NF; ++f)
+      for (int z = 0; z < NU; ++z) put(size_t(3 * NU + f) * w + col(z), lift(z, f));
+  } else {
+    constexpr int NT = G::NT, NL = G::NL, NQ = G::NQ;
+    std::vector<double> tv;
+    std::vector<int32_t> ti;
+    int pm = 0, pl = 0;
+    if (!build_prism_ops(R, tv, ti, &pm, &pl)) return false;
+    for (int t2 = 0; t2 < NT; ++t2)
+      for (int d = 0; d < 2; ++d)
+        for (int t = 0; t < NT; ++t)
+          put(size_t(t2 * 2 + d) * w + col(t), tv[size_t(d) * NT * NT + size_t(t) * NT + t2]);
+    for (int i = 0; i < NL * NL; ++i) o.B[i] = float(tv[size_t(2) * NT * NT + i]);
+    const size_t lq = size_t(2) * NT * w, lz = lq + size_t(NL) * NQ * w;
+    const size_t qf = m0c + size_t(NF) * nm, tf = qf + size_t(NL) * NQ;
+    std::vector<int> line(NF, -1), level(NF, -1);
+    for (int f = 0; f < NF; ++f)
+      for (int z = 0; z < NU; ++z) {
+        if (std::fabs(lift(z, f)) <= tl) continue;
+        int& own = f < 2 * NT ? line[f] : level[f];
+        const int i = f < 2 * NT ? z % NT : z / NT;
+        if (own >= 0 && own != i) return false;
+        own = i;
+      }
+    for (int a = 0; a < 2; ++a) {
+      std::vector<int> seen(NT, 0);
+      for (int f = a * NT; f < (a + 1) * NT; ++f) {
+        const int t = line[f];
+        if (t < 0 || seen[t]++) return false;
+        img[tf + size_t(a) * NT + t] = uint32_t(f);
+        for (int z = 0; z < NL; ++z) put(lz + (size_t(a) * NL + z) * NT + t, lift(z * NT + t, f));
+      }
+    }
+    for (int z = 0; z < NL; ++z) {
+      int j = 0;  // the level's flux points face by face, NL each
+      for (int f = 2 * NT; f < NF; ++f) {
+        if (level[f] < 0) return false;
+        if (level[f] != z) continue;
+        if (j >= NQ || face(f) != 2 + j / NL) return false;
+        img[qf + size_t(z) * NQ + j] = uint32_t(f);
+        for (int t = 0; t < NT; ++t)
+          put(lq + (size_t(z) * NQ + j) * w + col(t), lift(z * NT + t, f));
+        ++j;
+      }
+      if (j != NQ) return false;
+    }
+  }
+  for (int f = 0; f < NF; ++f) {
+    int j = 0;
+    for (int q = 0; q < NU; ++q) {
+      const double v = R.M0[size_t(f) * NU + q];
+      if (std::fabs(v) <= tm) continue;
+      put(m0v + size_t(f) * nm + j, v);
+      img[m0c + size_t(f) * nm + j] = uint32_t(q);
+      ++j;
+    }
+  }
   return true;
 }
 
@@ -728,7 +848,7 @@ int setup_device(fr_mesh* m) {
         D.m0_nm = nm;
       }
     }
-    if (D.kind == EK_PRI) {
+    if (D.kind == EK_PRI && sizeof(T) == 8) {
       std::vector<double> tv;
       std::vector<int32_t> ti;
       if (build_prism_ops(R, tv, ti, &D.pri_nm, &D.pri_nl)) {
@@ -748,6 +868,23 @@ int setup_device(fr_mesh* m) {
       }
     }
     if (sizeof(T) == 4 && D.kind != EK_HEX) {
+      std::vector<uint32_t> gi, vi;
+      dispatch(D.kind, m->order, [&](auto nu, auto nf) {
+        constexpr int NU = decltype(nu)::value, NF = decltype(nf)::value;
+        if constexpr (simplex_zb<NU, NF>(true) > 0)
+          D.sx_ok = build_simplex_ops<NU, NF>(R, simplex_zb<NU, NF>(true), gi, D.sx_grad) &&
+                    build_simplex_ops<NU, NF>(R, simplex_zb<NU, NF>(false), vi, D.sx_vol);
+      });
+      if (D.sx_ok) {
+        void *gd = nullptr, *vd = nullptr;
+        if ((rc = dev_zeros(m, gi.size() * 4, &gd)) || (rc = dev_zeros(m, vi.size() * 4, &vd)))
+          return rc;
+        CK(cudaMemcpy(gd, gi.data(), gi.size() * 4, cudaMemcpyHostToDevice));
+        CK(cudaMemcpy(vd, vi.data(), vi.size() * 4, cudaMemcpyHostToDevice));
+        D.sx_grad.img = static_cast<const float*>(gd);
+        D.sx_vol.img = static_cast<const float*>(vd);
+        D.pri_ok = D.kind == EK_PRI;
+      }
       bool fits = false;
       int tca = 0;
       bool order_ok = true;  // host face order = the compile-time one
@@ -943,12 +1080,6 @@ bool use_hex(const fr_mesh* m, const DevType& D) {
   return D.kind == EK_HEX && m->active != FR_VARIANT_DENSE;
 }
 
-// the viscous flux (9 values a point) is stored at the solution points in
-// place of the gradient (15), which the anti-aliased flux reads
-bool stores_visc(const fr_mesh* m, const DevType& D) {
-  return use_hex(m, D) && m->aa_qdeg == 0;
-}
-
 bool use_tc_grad(const fr_mesh* m, const DevType& D) {
   return D.tc_ok && D.tc_grad_on && m->active == FR_VARIANT_TENSOR;
 }
@@ -957,10 +1088,54 @@ bool use_tc_vol(const fr_mesh* m, const DevType& D) {
   return D.tc_ok && D.tc_vol_on && m->active == FR_VARIANT_TENSOR && m->aa_qdeg == 0;
 }
 
-// prisms on the structured kernels of fr_prism.cuh: every family but DENSE
-// (which keeps the dense operator products), no anti-aliasing
+// prisms on kernels that use their operators' structure (FP64: fr_prism.cuh,
+// FP32: fr_simplex.cuh): every family but DENSE (which keeps the dense
+// operator products), no anti-aliasing
 bool use_pri(const fr_mesh* m, const DevType& D) {
   return D.kind == EK_PRI && D.pri_ok && m->active != FR_VARIANT_DENSE && m->aa_qdeg == 0;
+}
+
+// the blocked FP32 kernels: tetrahedra and prisms outside the DENSE family
+// (which keeps the dense operator products), no anti-aliasing.  A type that
+// the tuner put on the tensor cores has both its kernels there: the blocked
+// ones hand the viscous flux from one to the other, the others the gradient.
+bool use_simplex(const fr_mesh* m, const DevType& D) {
+  return D.sx_ok && m->active != FR_VARIANT_DENSE && m->aa_qdeg == 0;
+}
+
+// the viscous flux (9 values a point) is stored at the solution points in
+// place of the gradient (15), which the anti-aliased flux and the
+// tensor-core kernels use
+bool stores_visc(const fr_mesh* m, const DevType& D) {
+  return (use_hex(m, D) && m->aa_qdeg == 0) || (use_simplex(m, D) && !use_tc_grad(m, D));
+}
+
+// elements per CTA of the blocked kernels: a thread per point, fewer where
+// that would leave SMs without a CTA (as dense_eb)
+template <int NU>
+int simplex_eb(long long ne, int num_sms) {
+  const long long per = (ne + num_sms - 1) / num_sms;
+  return int(std::min<long long>(simplex_threads<NU>() / NU,
+                                 std::max<long long>(per, (31 + NU) / NU)));
+}
+
+template <int NU, int NF>
+size_t simplex_smem(const DevType& D, int eb, bool grad) {
+  using G = SimplexGeom<NU, NF>;
+  const int nm = (grad ? D.sx_grad : D.sx_vol).nm;
+  return size_t(G::words(simplex_zb<NU, NF>(grad), nm) + eb * (grad ? G::kGrad : G::kVol)) * 4;
+}
+
+// their launch: grid and shared memory for the type's tile (CTAs per SM)
+template <int NU, int NF>
+void simplex_launch(const fr_mesh* m, const DevType& D, bool grad, int* eb, unsigned* grid,
+                    unsigned* threads, size_t* sm) {
+  *eb = simplex_eb<NU>(D.ne, m->num_sms);
+  *threads = unsigned((*eb * NU + 31) / 32 * 32);
+  *sm = simplex_smem<NU, NF>(D, *eb, grad);
+  const int mx = grad ? D.sx_grad_ctas : D.sx_vol_ctas, tile = grad ? D.tile_grad : D.tile_vol;
+  *grid = unsigned(std::min<long long>((D.ne + *eb - 1) / *eb,
+                                       (long long)m->num_sms * (tile > 0 && tile < mx ? tile : mx)));
 }
 
 template <typename T, int NU, int NF>
@@ -1158,9 +1333,9 @@ int prepare_kernels(fr_mesh* m) {
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kv1, E * NU, sv);
       D.grad_ctas = a > 0 ? a : 1;
       D.vol_ctas = b > 0 ? b : 1;
-      if constexpr (pri_order(NU, NF) > 0) {
+      if constexpr (sizeof(T) == 8 && pri_order(NU, NF) > 0) {
         if (D.pri_ok) {
-          auto pg = k_grad_pri<T, NU, NF, E, sizeof(T) == 4>;
+          auto pg = k_grad_pri<T, NU, NF, E>;
           auto pv0 = k_vol_pri<T, NU, NF, E, false>;
           auto pv1 = k_vol_pri<T, NU, NF, E, true>;
           const int psg = int(pri_grad_smem<T, NU, NF>(D)), psv = int(pri_vol_smem<T, NU, NF>(D));
@@ -1172,6 +1347,25 @@ int prepare_kernels(fr_mesh* m) {
           cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pb, pv1, E * NU, psv);
           D.pri_grad_ctas = pa > 0 ? pa : 1;
           D.pri_vol_ctas = pb > 0 ? pb : 1;
+        }
+      }
+      if constexpr (sizeof(T) == 4 && sizeof(TR) == 4 && simplex_zb<NU, NF>(true) > 0) {
+        if (D.sx_ok) {
+          constexpr int ZG = simplex_zb<NU, NF>(true), ZV = simplex_zb<NU, NF>(false);
+          const int eb = simplex_threads<NU>() / NU, th = simplex_threads<NU>();
+          const int smg = int(simplex_smem<NU, NF>(D, eb, true));
+          const int smv = int(simplex_smem<NU, NF>(D, eb, false));
+          auto xg = k_simplex_grad<NU, NF, ZG>;
+          auto xv0 = k_simplex_vol<NU, NF, ZV, false>;
+          auto xv1 = k_simplex_vol<NU, NF, ZV, true>;
+          cudaFuncSetAttribute(xg, cudaFuncAttributeMaxDynamicSharedMemorySize, smg);
+          cudaFuncSetAttribute(xv0, cudaFuncAttributeMaxDynamicSharedMemorySize, smv);
+          cudaFuncSetAttribute(xv1, cudaFuncAttributeMaxDynamicSharedMemorySize, smv);
+          int sa = 0, sb = 0;
+          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&sa, xg, th, smg);
+          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&sb, xv1, th, smv);
+          D.sx_grad_ctas = sa > 0 ? sa : 1;
+          D.sx_vol_ctas = sb > 0 ? sb : 1;
         }
       }
       if constexpr (tc_types<T, TR>() && tc_supported<NU, NF>()) {
@@ -1319,8 +1513,9 @@ inline std::vector<int> tile_candidates(const fr_mesh* m, const DevType& D, bool
       if (k == 1) break;
     }
   } else {
-    const int mx = use_pri(m, D) ? (grad ? D.pri_grad_ctas : D.pri_vol_ctas)
-                                 : (grad ? D.grad_ctas : D.vol_ctas);
+    const int mx = use_simplex(m, D) ? (grad ? D.sx_grad_ctas : D.sx_vol_ctas)
+                   : use_pri(m, D)   ? (grad ? D.pri_grad_ctas : D.pri_vol_ctas)
+                                     : (grad ? D.grad_ctas : D.vol_ctas);
     for (int k = mx; k >= 1; k /= 2) c.push_back(k);
   }
   return c;
@@ -1500,16 +1695,31 @@ void launch_stage(fr_mesh* m, cudaStream_t s, int mode, int stage,
         });
       } else if (use_tc_grad(m, D)) {
         launch_grad_tc<T, TR>(m, D, s, from_x, du, va, bc, ph);
+      } else if (use_simplex(m, D)) {
+        dispatch(D.kind, m->order, [&](auto nu, auto nf) {
+          constexpr int NU = decltype(nu)::value, NF = decltype(nf)::value;
+          if constexpr (sizeof(T) == 4 && sizeof(TR) == 4 && simplex_zb<NU, NF>(true) > 0) {
+            constexpr int ZB = simplex_zb<NU, NF>(true);
+            int eb;
+            unsigned grid, th;
+            size_t sm;
+            simplex_launch<NU, NF>(m, D, true, &eb, &grid, &th, &sm);
+            const T* uin = from_x ? (const T*)D.X : (const T*)D.Y;
+            k_simplex_grad<NU, NF, ZB><<<grid, th, sm, s>>>(
+                D.ne, eb, uin, ta, (const T*)D.smat, (const T*)D.rcpdjac, D.sx_grad,
+                (T*)D.grad, va, bc, ph);
+          }
+        });
       } else if (use_pri(m, D)) {
         dispatch(D.kind, m->order, [&](auto nu, auto nf) {
           constexpr int NU = decltype(nu)::value, NF = decltype(nf)::value;
-          if constexpr (pri_order(NU, NF) > 0) {
+          if constexpr (sizeof(T) == 8 && pri_order(NU, NF) > 0) {
             constexpr int E = dense_epb<NU>();
             const int eb = dense_eb<NU>(D.ne, m->num_sms);
             const unsigned grid = unsigned(std::min<long long>(
                 (D.ne + eb - 1) / eb,
                 (long long)m->num_sms * (D.tile_grad > 0 ? D.tile_grad : D.pri_grad_ctas)));
-            k_grad_pri<T, NU, NF, E, sizeof(T) == 4>
+            k_grad_pri<T, NU, NF, E>
                 <<<grid, eb * NU, pri_grad_smem<T, NU, NF>(D, eb), s>>>(
                     D.ne, eb, from_x ? (const T*)D.X : (const T*)D.Y, ta, (const T*)D.smat,
                     (const T*)D.rcpdjac, pri_ops_of<T>(m, D), (T*)D.grad, va, bc, ph);
@@ -1646,10 +1856,32 @@ void launch_stage(fr_mesh* m, cudaStream_t s, int mode, int stage,
       sa.uf_next = uf_next;
       sa.E = m->err_on ? (T*)D.E : nullptr;
       const T* uin = from_x ? (const T*)D.X : (const T*)D.Y;
-      if (use_pri(m, D)) {
+      if (use_simplex(m, D)) {
         dispatch(D.kind, m->order, [&](auto nu, auto nf) {
           constexpr int NU = decltype(nu)::value, NF = decltype(nf)::value;
-          if constexpr (pri_order(NU, NF) > 0) {
+          if constexpr (sizeof(T) == 4 && sizeof(TR) == 4 && simplex_zb<NU, NF>(false) > 0) {
+            constexpr int ZB = simplex_zb<NU, NF>(false);
+            int eb;
+            unsigned grid, th;
+            size_t sm;
+            simplex_launch<NU, NF>(m, D, false, &eb, &grid, &th, &sm);
+            HexStage<T, TR> ha{mode, stage, (TR*)D.X, (TR*)D.A, (T*)D.Y, (T*)D.R,
+                               m->d_dt, m->d_flag, uf_next};
+            ha.E = m->err_on ? (TR*)D.E : nullptr;
+            if (ns)
+              k_simplex_vol<NU, NF, ZB, true><<<grid, th, sm, s>>>(
+                  D.ne, eb, uin, (const T*)D.grad, fc, (const T*)D.smat, (const T*)D.rcpdjac,
+                  D.sx_vol, ph, ha);
+            else
+              k_simplex_vol<NU, NF, ZB, false><<<grid, th, sm, s>>>(
+                  D.ne, eb, uin, nullptr, fc, (const T*)D.smat, (const T*)D.rcpdjac, D.sx_vol,
+                  ph, ha);
+          }
+        });
+      } else if (use_pri(m, D)) {
+        dispatch(D.kind, m->order, [&](auto nu, auto nf) {
+          constexpr int NU = decltype(nu)::value, NF = decltype(nf)::value;
+          if constexpr (sizeof(T) == 8 && pri_order(NU, NF) > 0) {
             constexpr int E = dense_epb<NU>();
             const int eb = dense_eb<NU>(D.ne, m->num_sms);
             const unsigned grid = unsigned(std::min<long long>(
@@ -1994,16 +2226,17 @@ int resolve_variant(fr_mesh* m, int scheme, double dt) {
     }
   }
   if (has_tc) {
-    // tensor cores only for the kernels (gradient, volume) of the types that
-    // ran faster there; re-time the tensor family with that choice
+    // tensor cores only for the types whose gradient and volume kernel
+    // together ran faster there (what one hands to the other differs, see
+    // stores_visc); re-time the tensor family with that choice
     bool any = false, all = true;
     for (size_t t = 0; t < nt; ++t) {
       DevType& D = m->types[t];
       if (!D.tc_ok) continue;
-      D.tc_grad_on = t_tc[2 * t] < t_cc[2 * t];
-      D.tc_vol_on = t_tc[2 * t + 1] < t_cc[2 * t + 1];
-      any |= D.tc_grad_on || D.tc_vol_on;
-      all &= D.tc_grad_on && D.tc_vol_on;
+      D.tc_grad_on = D.tc_vol_on =
+          t_tc[2 * t] + t_tc[2 * t + 1] < t_cc[2 * t] + t_cc[2 * t + 1];
+      any |= D.tc_grad_on;
+      all &= D.tc_grad_on;
     }
     if (!any) {
       if (pick == FR_VARIANT_TENSOR) {  // no type gains: best CUDA-core family

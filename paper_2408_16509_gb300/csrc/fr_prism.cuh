@@ -1,4 +1,5 @@
-// Prism kernels that use the structure of the prism's operators (Section 3.1,
+// FP64 prism kernels (FP32: fr_simplex.cuh) that use the structure of the
+// prism's operators (Section 3.1,
 // "Matrix multiplications": the operator matrices are sparse, and kernels
 // that skip their zeros do less work than dense products).
 //
@@ -98,8 +99,8 @@ __device__ __forceinline__ PriOps<T> stage_pri_ops(const PriOps<T>& g, unsigned 
 
 // NS gradient path on prisms (as k_grad_dense): corrected reference
 // gradient, physical gradient at the solution points (global and shared),
-// its values at the flux points (q form: the viscous normal flux there).
-template <typename T, int NU, int NF, int EPB, bool QV>
+// its values at the flux points.
+template <typename T, int NU, int NF, int EPB>
 __global__ void __launch_bounds__(EPB* NU)
     k_grad_pri(long long ne, int eb, const T* __restrict__ u,
                const __grid_constant__ TraceArgs<T> ta,
@@ -202,12 +203,8 @@ __global__ void __launch_bounds__(EPB* NU)
 #pragma unroll
           for (int c = 0; c < 15; ++c) acc[c] += m * g[c];
         }
-        if (QV) {
-          write_visc_q(va, bc, ph, e, f, NF, acc);
-        } else {
 #pragma unroll
-          for (int c = 0; c < 15; ++c) va.q[(e * 15 + c) * NF + f] = acc[c];
-        }
+        for (int c = 0; c < 15; ++c) va.q[(e * 15 + c) * NF + f] = acc[c];
       }
     }
     __syncthreads();
