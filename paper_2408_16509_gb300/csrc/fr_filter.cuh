@@ -69,8 +69,19 @@ struct FilterOps {
   const int32_t* partner;  // [ne][nf] partner flux-point code or -1
 };
 
+// threads of a CTA of the kernels that take an element per warp
+constexpr int kScanThreads = 128;
+
+// gamma for the FP32 screens and the double-float selections, prepared on the
+// host (in the kernels they were some ten FP64 instructions a warp)
+struct GammaArgs {
+  float g, gm1h, gm1l;  // gamma; gamma - 1 as a double-float
+  bool by5;             // entropy_by_s5
+};
+
 struct FilterArgs {
   double gamma;
+  GammaArgs gf;
   double tau;            // relative entropy tolerance
   double ratio;          // first bracket step around a predicted guess
   float* zeta_last;      // [ne] zeta of the last filtered stage (0: none)
@@ -93,7 +104,7 @@ struct FilterArgs {
 // relative; FP64 1.4 itself is 7/5 to 6e-17).  y is formed only where it
 // stays a normal FP64 number (s5_in_range); other points take the
 // per-point pow.
-__device__ __forceinline__ bool entropy_by_s5(double g) { return g == 1.4; }
+inline bool entropy_by_s5(double g) { return g == 1.4; }
 
 // unbiased binary exponent of x from its bits (integer pipe)
 __device__ __forceinline__ int dexp2(double x) {
@@ -207,25 +218,157 @@ __device__ __forceinline__ double warp_sum(double v) {
 // of least entropy; its FP64 value is left to k_entropy_value, where a warp
 // evaluates 32 elements at once (here one lane would hold the warp for some
 // 50 FP64 instructions of 64 clocks each): 16384 FP32 hexahedra of order 3,
-// 106 -> 59 + 6 us.
+// 106 -> 41 + 6 us.
 struct EntropyRec {
   float v[5];  // the selected point's state; v[0] = 0: none
   float pad;
   double m;    // minimum over points that took the per-point pow
 };
 
+// The warp's part of k_entropy_min for FP32 values and gamma = 7/5: the point
+// of least s^5 by double-float arithmetic (FP64 where the pressure is too
+// close to zero to sign), its state to the record.  All loads go out before
+// the first screen: with a load, a screen and a branch per slot the warp
+// waited for each slot's latency in turn (16384 hexahedra of order 3: 59 ->
+// 41 us; 8.5 of 12 stalled warps waited for loads).
+template <int NU, int NF>
+__device__ __forceinline__ void entropy_select(long long e, const float* __restrict__ u,
+                                               const float* __restrict__ uf,
+                                               const float* __restrict__ uf_all,
+                                               const TypeTab& tt,
+                                               const int32_t* __restrict__ partner,
+                                               double gamma, const GammaArgs& gc,
+                                               EntropyRec* __restrict__ rec) {
+  constexpr int NQ = (NU + 2 * NF + 31) / 32;
+  const int lane = threadIdx.x & 31;
+  float v[NQ][5], slo[NQ];
+  int32_t code[NQ];
+  uint32_t have = 0, cand = 0;  // bit q: slot q holds a point / needs the comparison
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) {
+    const int i = lane + 32 * q;
+    code[q] = i >= NU + NF && i < NU + 2 * NF ? partner[e * NF + (i - NU - NF)] : -1;
+  }
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) {
+    const int i = lane + 32 * q;
+    const float* p = i < NU ? u + e * 5 * NU + i : uf + e * 5 * NF + (i - NU);
+    int st = i < NU ? NU : NF;
+    if (code[q] >= 0) {
+      const FluxPt c(code[q], tt);
+      p = uf_all + c.p5;
+      st = c.nf;
+    }
+    const bool ok = i < NU + NF || code[q] >= 0;
+    have |= uint32_t(ok) << q;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) v[q][k] = ok ? p[(long long)k * st] : 0.f;
+  }
+  float shi_min = INFINITY;
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) {
+    slo[q] = INFINITY;
+    if (!((have >> q) & 1u)) continue;
+    const PtScreen sc = screen_point(v[q][0], v[q][1], v[q][2], v[q][3], v[q][4], gc.g);
+    if (!sc.pos || sc.phi <= 0.f) continue;  // not admissible
+    if (sc.plo <= 0.f) {                     // admissibility undecided
+      cand |= 1u << q;
+      continue;
+    }
+    slo[q] = sc.slo;
+    shi_min = fminf(shi_min, sc.shi);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+    shi_min = fminf(shi_min, __shfl_xor_sync(0xffffffffu, shi_min, o));
+  const dfl gm1d{gc.gm1h, gc.gm1l};
+  constexpr long long kNone = 0x7fffffffffffffffLL;
+  double m = INFINITY;  // direct minimum (points outside the s^5 range)
+  long long ky = kNone;
+  int qy = -1;
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) {
+    if (!((have >> q) & 1u) || (!((cand >> q) & 1u) && !(slo[q] <= shi_min))) continue;
+    const float* vf = v[q];
+    if (!(vf[0] > 0.f)) continue;
+    bool amb = !(vf[0] >= 0x1p-100f && vf[0] <= 0x1p100f);
+    dfl rr{0.f, 0.f}, pd{0.f, 0.f};
+    if (!amb) {
+      rr = df_rcp(vf[0]);
+      pd = df_pressure(vf[1], vf[2], vf[3], vf[4], rr, gm1d, &amb);
+    }
+    long long yk = 0;
+    bool ykey = false;
+    if (amb) {
+      double w[5];
+#pragma unroll
+      for (int k = 0; k < 5; ++k) w[k] = widen_f32(vf[k]);
+      const double rr64 = rcp64(w[0], vf[0]);
+      const double p = (gamma - 1.0) * (w[4] - 0.5 * (w[1] * w[1] + w[2] * w[2] + w[3] * w[3]) * rr64);
+      if (!(p > 0.0)) continue;
+      if (s5_in_range(p, rr64)) {
+        yk = key47_f64(s5_of(p, rr64));
+        ykey = true;
+      } else {
+        m = dmin_key(m, p * pow(w[0], -gamma));
+      }
+    } else {
+      if (!(pd.hi > 0.f)) continue;
+      if (df_s5_key(pd, rr, &yk)) {
+        ykey = true;
+      } else {
+        double w[5];
+#pragma unroll
+        for (int k = 0; k < 5; ++k) w[k] = widen_f32(vf[k]);
+        m = dmin_key(m, pressure64(w, gamma) * pow(w[0], -gamma));
+      }
+    }
+    if (ykey) {
+      const long long kt = (yk << 5) | lane;
+      if (kt < ky) {
+        ky = kt;
+        qy = q;
+      }
+    }
+  }
+  long long km = dkey(m), kym = ky;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    km = min(km, __shfl_xor_sync(0xffffffffu, km, o));
+    kym = min(kym, __shfl_xor_sync(0xffffffffu, kym, o));
+  }
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) {  // one lane: keys carry the lane
+    if (qy == q && ky == kym) {
+#pragma unroll
+      for (int k = 0; k < 5; ++k) rec->v[k] = v[q][k];
+    }
+  }
+  if (lane == 0) {
+    rec->m = dunkey(km);
+    if (kym == kNone) rec->v[0] = 0.f;
+  }
+}
+
 template <typename T, typename TR, int NU, int NF>
-__global__ void k_entropy_min(long long ne, const T* __restrict__ uin,
+__global__ void __launch_bounds__(kScanThreads, (NU + 2 * NF + 31) / 32 <= 8 ? 5 : 4)
+    k_entropy_min(long long ne, const T* __restrict__ uin,
                               const TR* __restrict__ X,
                               const T* __restrict__ uf_all, TypeTab tt,
                               int tidx, const int32_t* __restrict__ partner,
-                              double gamma, double* __restrict__ smin,
+                              double gamma, GammaArgs gc, double* __restrict__ smin,
                               EntropyRec* __restrict__ rec) {
   constexpr int NQ = (NU + 2 * NF + 31) / 32;
   const int lane = threadIdx.x & 31;
   const long long e = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (e >= ne) return;
   const T* uf = uf_all + tt.off_f[tidx];
+  if constexpr (sizeof(T) == 4 && sizeof(TR) == 4) {
+    if (gc.by5) {
+      entropy_select<NU, NF>(e, uin ? uin : X, uf, uf_all, tt, partner, gamma, gc, rec + e);
+      return;
+    }
+  }
   // state at point slot i, converted to V (float for the screen, double
   // for the exact value); false when the slot holds no point
   auto load = [&](int i, auto* v) -> bool {
@@ -252,7 +395,7 @@ __global__ void k_entropy_min(long long ne, const T* __restrict__ uin,
     }
     return false;
   };
-  const float gf = float(gamma);
+  const float gf = gc.g;
   float slo[NQ];
   uint32_t cand = 0;  // bit q: slot q needs the FP64 value
   float shi_min = INFINITY;
@@ -278,85 +421,10 @@ __global__ void k_entropy_min(long long ne, const T* __restrict__ uin,
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1)
     shi_min = fminf(shi_min, __shfl_xor_sync(0xffffffffu, shi_min, o));
-  const bool by5 = entropy_by_s5(gamma);
+  const bool by5 = gc.by5;
   // the stored values as FP64: FP32 stage values widened exactly on the
   // integer pipe (the FP64 pipe is this kernel's bound)
   constexpr bool f32in = sizeof(T) == 4 && sizeof(TR) == 4;
-  if constexpr (f32in) {
-    if (by5) {
-      // FP32 values, gamma = 7/5: the point of least s^5 is selected in
-      // double-float arithmetic (FP64 where the pressure is too close to
-      // zero to sign), then s^5 is computed in FP64 at that point
-      const float gm1h = float(gamma - 1.0);
-      const dfl gm1d{gm1h, float((gamma - 1.0) - widen_f32(gm1h))};
-      double m = INFINITY;  // direct minimum (points outside the s^5 range)
-      long long ky = 0x7fffffffffffffffLL;
-      int qy = -1;
-#pragma unroll
-      for (int q = 0; q < NQ; ++q) {
-        if (!((cand >> q) & 1u) && !(slo[q] <= shi_min)) continue;
-        float vf[5];
-        if (!load(lane + 32 * q, vf)) continue;
-        if (!(vf[0] > 0.f)) continue;
-        bool amb = !(vf[0] >= 0x1p-100f && vf[0] <= 0x1p100f);
-        dfl rr{0.f, 0.f}, pd{0.f, 0.f};
-        if (!amb) {
-          rr = df_rcp(vf[0]);
-          pd = df_pressure(vf[1], vf[2], vf[3], vf[4], rr, gm1d, &amb);
-        }
-        long long yk = 0;
-        bool ykey = false;
-        if (amb) {
-          double v[5];
-#pragma unroll
-          for (int k = 0; k < 5; ++k) v[k] = widen_f32(vf[k]);
-          const double rr64 = rcp64(v[0], vf[0]);
-          const double p = (gamma - 1.0) * (v[4] - 0.5 * (v[1] * v[1] + v[2] * v[2] + v[3] * v[3]) * rr64);
-          if (!(p > 0.0)) continue;
-          if (s5_in_range(p, rr64)) {
-            yk = key47_f64(s5_of(p, rr64));
-            ykey = true;
-          } else {
-            m = dmin_key(m, p * pow(v[0], -gamma));
-          }
-        } else {
-          if (!(pd.hi > 0.f)) continue;
-          if (df_s5_key(pd, rr, &yk)) {
-            ykey = true;
-          } else {
-            double v[5];
-#pragma unroll
-            for (int k = 0; k < 5; ++k) v[k] = widen_f32(vf[k]);
-            m = dmin_key(m, pressure64(v, gamma) * pow(v[0], -gamma));
-          }
-        }
-        if (ykey) {
-          const long long kt = (yk << 5) | lane;
-          if (kt < ky) {
-            ky = kt;
-            qy = q;
-          }
-        }
-      }
-      long long km = dkey(m), kym = ky;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        km = min(km, __shfl_xor_sync(0xffffffffu, km, o));
-        kym = min(kym, __shfl_xor_sync(0xffffffffu, kym, o));
-      }
-      if (qy >= 0 && ky == kym) {  // one lane: keys carry the lane
-        float vf[5];
-        load(lane + 32 * qy, vf);
-#pragma unroll
-        for (int k = 0; k < 5; ++k) rec[e].v[k] = vf[k];
-      }
-      if (lane == 0) {
-        rec[e].m = dunkey(km);
-        if (kym == 0x7fffffffffffffffLL) rec[e].v[0] = 0.f;
-      }
-      return;
-    }
-  }
   double m = INFINITY, y = INFINITY;  // direct minimum, minimum of s^5
 #pragma unroll
   for (int q = 0; q < NQ; ++q) {
@@ -635,7 +703,8 @@ __device__ __forceinline__ void warp_minima(const T (&v)[NQ][5], const PtScreen 
 // FP32 values: the points that decide an element's zeta = 0 test, selected by
 // a warp (as warp_minima, in double-float arithmetic where gamma = 7/5),
 // evaluated in FP64 by k_filter_decide, a thread per element (16384
-// hexahedra of order 3: 139 -> 56 + 6 us against a warp that did both).
+// hexahedra of order 3: 139 -> 33 + 6 us against a warp that did both; with
+// its loads all before the screens and gamma's constants from the host 56 -> 33).
 struct CheckRec {
   float pv[5];  // point of least pressure; has & 1
   float yv[5];  // point of least s^5; has & 2
@@ -805,7 +874,8 @@ static __global__ void k_filter_decide(long long ne, const CheckRec* __restrict_
 // are left alone (zeta 0, one evaluation); the others are listed for
 // k_filter, which takes the oracle's modal form from there.
 template <typename T, typename TR, int NU, int NF>
-__global__ void k_filter_check(long long ne, const T* __restrict__ reg,
+__global__ void __launch_bounds__(kScanThreads, (NU + NF + 31) / 32 <= 8 ? 5 : 4)
+    k_filter_check(long long ne, const T* __restrict__ reg,
                                const TR* __restrict__ regR, const T* __restrict__ uf,
                                FilterArgs fa, int32_t* __restrict__ list,
                                int* __restrict__ count, CheckRec* __restrict__ rec) {
@@ -814,34 +884,38 @@ __global__ void k_filter_check(long long ne, const T* __restrict__ reg,
   const long long e = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (e >= ne) return;  // whole warps
   const double g = fa.gamma;
-  const float gf = float(g);
-  const bool by5 = entropy_by_s5(g);
-  const float gm1h = float(g - 1.0);
-  const dfl gm1d{gm1h, float((g - 1.0) - widen_f32(gm1h))};
   const double smin = fa.smin[e];
-  const double sb = smin * (1.0 - fa.tau);
   T v[NQ][5];
   PtScreen sc[NQ];
 #pragma unroll
-  for (int q = 0; q < NQ; ++q) {
+  for (int q = 0; q < NQ; ++q) {  // all loads before the first screen
     const int i = lane + 32 * q;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+      v[q][k] = T(0);
+      if (i < NU)
+        v[q][k] = reg ? reg[(e * 5 + k) * NU + i] : T(regR[(e * 5 + k) * NU + i]);
+      else if (i < NP)
+        v[q][k] = uf[(e * 5 + k) * NF + (i - NU)];
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) {
     sc[q].pos = false;
     sc[q].plo = sc[q].slo = INFINITY;
-#pragma unroll
-    for (int k = 0; k < 5; ++k) v[q][k] = T(0);
-    if (i >= NP) continue;
-#pragma unroll
-    for (int k = 0; k < 5; ++k)
-      v[q][k] = i < NU ? (reg ? reg[(e * 5 + k) * NU + i] : T(regR[(e * 5 + k) * NU + i]))
-                       : uf[(e * 5 + k) * NF + (i - NU)];
-    sc[q] = screen_point(float(v[q][0]), float(v[q][1]), float(v[q][2]), float(v[q][3]),
-                         float(v[q][4]), gf);
+    if (lane + 32 * q < NP)
+      sc[q] = screen_point(float(v[q][0]), float(v[q][1]), float(v[q][2]), float(v[q][3]),
+                           float(v[q][4]), fa.gf.g);
   }
   if constexpr (sizeof(T) == 4) {
-    warp_select<NQ, NP>(v, sc, smin > 0.0, g, by5, gm1d, rec + e);
+    // smin > 0 without an FP64 comparison (NaN: false)
+    const long long sbits = __double_as_longlong(smin);
+    warp_select<NQ, NP>(v, sc, sbits > 0 && sbits <= 0x7ff0000000000000LL, g, fa.gf.by5,
+                        dfl{fa.gf.gm1h, fa.gf.gm1l}, rec + e);
   } else {
+    const double sb = smin * (1.0 - fa.tau);
     double r, p, sdir, ys;
-    warp_minima<T, NQ, NP>(v, sc, smin, g, by5, &r, &p, &sdir, &ys);
+    warp_minima<T, NQ, NP>(v, sc, smin, g, fa.gf.by5, &r, &p, &sdir, &ys);
     if (lane == 0) check_outcome(e, r, p, sdir, ys, smin, sb, fa, list, count);
   }
 }
@@ -882,11 +956,12 @@ __device__ __forceinline__ void filter_element(const long long e, T* __restrict_
   __shared__ double s_z;        // requested strength
   const int tid = threadIdx.x;
   const double g = fa.gamma;
-  const float gf = float(g);
-  const bool by5 = entropy_by_s5(g);
-  const float gm1h = float(g - 1.0);
-  const dfl gm1d{gm1h, float((g - 1.0) - widen_f32(gm1h))};  // gamma - 1, double-float
-  __shared__ double s_sel[3];  // FP64 values at the selected points
+  const float gf = fa.gf.g;
+  const bool by5 = fa.gf.by5;
+  const dfl gm1d{fa.gf.gm1h, fa.gf.gm1l};  // gamma - 1, double-float
+  __shared__ double s_sel[4];   // FP64 values at the selected points
+  __shared__ float s_pt[2][5];  // their states
+  __shared__ float s_zf[2];     // the strength as a double-float
   __shared__ T us[5][NU];
   const double smin = fa.smin[e];
   const double sb = smin * (1.0 - fa.tau);
@@ -900,15 +975,24 @@ __device__ __forceinline__ void filter_element(const long long e, T* __restrict_
   struct Mins {
     double r, p, s;  // s: minimum over the points that took the per-point pow
     double ys;       // minimum of s^5 over the others (entropy_by_s5)
+    double sm;       // FP32 values: the least s of all, on thread 0's warp
   };
-  // the entropy minimum of an evaluation (one pow, by the thread that needs it)
-  auto smin_of = [](const Mins& q) -> double {
+  // the entropy minimum of an evaluation (one fifth root, by the thread that
+  // needs it; by5 with FP32 values: already in sm)
+  auto smin_of = [&](const Mins& q) -> double {
+    if (sizeof(T) == 4 && by5) return q.sm;
     return q.ys < INFINITY ? fmin(q.s, s_of_s5(q.ys)) : q.s;
   };
   auto minima = [&](double z) -> Mins {
     for (int m = tid; m < NM; m += kFilterThreads) {
-      double d = double(op.deg[m]);
-      const T sk = sizeof(T) == 4 ? T(__expf(-float(z * d * d))) : T(exp(-z * d * d));
+      T sk;
+      if constexpr (sizeof(T) == 4) {  // z d^2 from the halves of both, no FP64
+        const float d = op.deg[m], d2 = d * d, d2l = fmaf(d, d, -d2);
+        sk = __expf(-fmaf(s_zf[0], d2, fmaf(s_zf[0], d2l, s_zf[1] * d2)));
+      } else {
+        const double d = double(op.deg[m]);
+        sk = T(exp(-z * d * d));
+      }
 #pragma unroll
       for (int k = 0; k < 5; ++k) ush[m][k] = sk * uh[k][m];
     }
@@ -1017,28 +1101,43 @@ __device__ __forceinline__ void filter_element(const long long e, T* __restrict_
         block_min_ll4(kr, kpm, kms, kym, redk);
         rmin = dunkey(kr);
         ms = dunkey(kms);
-        // the selected points' FP64 values (one writer each)
+        // the selected points' FP64 values, each by a warp of its own: a
+        // chain of some twenty (p) and fifty (s) dependent FP64 instructions
         if (qp >= 0 && kp == kpm) {
-          double w[5];
 #pragma unroll
-          for (int k = 0; k < 5; ++k) w[k] = to_f64(v[qp][k]);
-          s_sel[0] = pressure64(w, g);
+          for (int k = 0; k < 5; ++k) s_pt[0][k] = v[qp][k];
         }
         if (qy >= 0 && ky == kym) {
-          double w[5];
 #pragma unroll
-          for (int k = 0; k < 5; ++k) w[k] = to_f64(v[qy][k]);
-          const double rr64 = rcp64(w[0], float(v[qy][0]));
-          const double p64 = (g - 1.0) * (w[4] - 0.5 * (w[1] * w[1] + w[2] * w[2] + w[3] * w[3]) * rr64);
-          s_sel[1] = s5_in_range(p64, rr64) ? s5_of(p64, rr64) : INFINITY;
-          if (!s5_in_range(p64, rr64)) s_sel[2] = p64 * pow(w[0], -g);
+          for (int k = 0; k < 5; ++k) s_pt[1][k] = v[qy][k];
         }
         __syncthreads();
-        mp = kpm == 0x7fffffffffffffffLL ? INFINITY : s_sel[0];
-        ys = kym == 0x7fffffffffffffffLL ? INFINITY : s_sel[1];
-        if (kym != 0x7fffffffffffffffLL && !(s_sel[1] < INFINITY)) ms = fmin(ms, s_sel[2]);
+        constexpr long long kNone = 0x7fffffffffffffffLL;
+        if (tid == 32 && kpm != kNone) {
+          double w[5];
+#pragma unroll
+          for (int k = 0; k < 5; ++k) w[k] = to_f64(s_pt[0][k]);
+          s_sel[0] = pressure64(w, g);
+        }
+        if (tid == 64) {
+          double sd = ms, y = INFINITY;
+          if (kym != kNone) {
+            double w[5];
+#pragma unroll
+            for (int k = 0; k < 5; ++k) w[k] = to_f64(s_pt[1][k]);
+            const double rr64 = rcp64(w[0], s_pt[1][0]);
+            const double p64 = (g - 1.0) * (w[4] - 0.5 * (w[1] * w[1] + w[2] * w[2] + w[3] * w[3]) * rr64);
+            if (s5_in_range(p64, rr64)) y = s5_of(p64, rr64);
+            else sd = fmin(sd, p64 * pow(w[0], -g));
+          }
+          s_sel[1] = y;
+          s_sel[2] = sd;
+          s_sel[3] = y < INFINITY ? fmin(sd, s_of_s5(y)) : sd;
+        }
+        __syncthreads();
+        mp = kpm == kNone ? INFINITY : s_sel[0];
         // (s_sel is written again only after the next evaluation's barriers)
-        return Mins{rmin, mp, ms, ys};
+        return Mins{rmin, mp, s_sel[2], s_sel[1], s_sel[3]};
       }
     }
 #pragma unroll
@@ -1069,7 +1168,7 @@ __device__ __forceinline__ void filter_element(const long long e, T* __restrict_
       }
     }
     block_min4_key(rmin, mp, ms, ys, redk);
-    return Mins{rmin, mp, ms, ys};
+    return Mins{rmin, mp, ms, ys, 0.0};
   };
   // unfiltered state admissible (the sign of the margin below, which the
   // positive means do not change): nothing to do (uniform across the block).
@@ -1107,35 +1206,26 @@ __device__ __forceinline__ void filter_element(const long long e, T* __restrict_
 #pragma unroll
     for (int k = 0; k < 5; ++k) uh[k][m] = acc[k];
   }
-  // the same test on the modal evaluation (the oracle's form)
-  Mins m0 = minima(0.0);
-  if (admissible(m0)) {
-    leave_unfiltered();
-    return;
-  }
-  // a filtered element: its entropy minimum at z = 0 (one pow, warp 0:
-  // the predictor's features and thread 0's margin read it)
-  if (tid < 32) m0.s = smin_of(m0);
-  m0.ys = INFINITY;
-  // element means of density and pressure (normalise the margin)
-  double wr = 0.0, wp = 0.0, ws = 0.0;
-  for (int z = tid; z < NU; z += kFilterThreads) {
-    const double w5[5] = {double(us[0][z]), double(us[1][z]), double(us[2][z]),
-                          double(us[3][z]), double(us[4][z])};
-    const double p = pressure64(w5, g);
-    double w = double(op.W[z]);
-    wr += w * double(us[0][z]);
-    wp += w * p;
-    ws += w;
-  }
-  const double wsum = block_sum(ws, red);
-  const double rmean = fmax(block_sum(wr, red) / wsum, kEpsPos);
-  const double pmean = fmax(block_sum(wp, red) / wsum, kEpsPos);
+  if (tid == 0) s_zf[0] = s_zf[1] = 0.f;
+  __syncthreads();
+  // ---- One call of minima, in a loop whose first pass is the unfiltered
+  // state: the code is fetched anew at every launch, a second copy of it too.
+  // Root-find:  Thread 0 runs the bracketing and Illinois logic as a
+  // state machine and publishes the next strength in shared memory; every
+  // evaluation of the margin is a block operation.
+  enum { kPlainHi = 0, kGuess = 1, kDown = 2, kUp = 3, kIllinois = 4, kDone = 5 };
+  __shared__ double s_next;
+  __shared__ int s_go;
+  // ghr: the margin at hi (ghi is halved by the Illinois rule)
+  double lo = 0.0, glo = 0.0, hi = kZetaMax, ghi = 0.0, ghr = 0.0, result = 0.0, zc = 0.0;
+  int evals = 1, state = kPlainHi, it = 0, side = 0;
+  bool fallback = false, use_guess = false;
+  float feat[4] = {0.f, 0.f, 0.f, 0.f};
+  double rmean = 0.0, pmean = 0.0, irm = 0.0, ipm = 0.0, ism = 0.0;
   // margin g(z) = min((rho-eps)/rho_mean, (p-eps)/p_mean, (s-sb)/s_min); one
   // thread evaluates it, a chain of FP64 instructions of 64 clocks each: the
   // divisors are inverted once for FP32 values (FP64 values keep the oracle's
   // divisions, whose evaluation counts they reproduce)
-  const double irm = 1.0 / rmean, ipm = 1.0 / pmean, ism = smin > 0.0 ? 1.0 / smin : 0.0;
   auto gval = [&](const Mins& q) -> double {
     double gr, gp, gs = INFINITY;
     if constexpr (sizeof(T) == 4) {
@@ -1151,51 +1241,6 @@ __device__ __forceinline__ void filter_element(const long long e, T* __restrict_
     if (isnan(gm)) gm = -INFINITY;
     return gm;
   };
-  auto margin = [&](double z) -> double { return gval(minima(z)); };
-  // predictor inputs from the unfiltered state (z = 0)
-  float feat[4] = {0.f, 0.f, 0.f, 0.f};
-  if (fa.mlp || fa.samples) {
-    double eh = 0.0, et = 0.0;
-    for (int m = tid; m < NM; m += kFilterThreads) {
-      double d = double(op.deg[m]), c = double(uh[0][m]);
-      if (d > 1.0) eh += c * c;
-      if (d > 0.0) et += c * c;
-    }
-    eh = block_sum(eh, red);
-    et = block_sum(et, red);
-    feat[0] = float(fmin(fmax(log10((eh + 1e-30) / (et + 1e-30)), -30.0), 30.0));
-    feat[1] = float(fmin(fmax(m0.r / rmean, -30.0), 30.0));
-    feat[2] = float(fmin(fmax(m0.p / pmean, -30.0), 30.0));
-    // log10 of the entropy-bound violation (floor 1e-14)
-    double f3 = 1.0;
-    if (smin > 0.0 && m0.s > -INFINITY && m0.r > 0.0 && m0.p > 0.0)
-      f3 = fmax((smin - m0.s) / smin, 1e-14);
-    feat[3] = float(log10(f3));
-  }
-  const double g0 = gval(m0);
-  // ---- root-find.  Thread 0 runs the bracketing and Illinois logic as a
-  // state machine and publishes the next strength in shared memory; every
-  // evaluation of the margin is a block operation.
-  enum { kPlainHi = 0, kGuess = 1, kDown = 2, kUp = 3, kIllinois = 4, kDone = 5 };
-  __shared__ double s_next;
-  __shared__ int s_go;
-  // ghr: the margin at hi (ghi is halved by the Illinois rule)
-  double lo = 0.0, glo = g0, hi = kZetaMax, ghi = 0.0, ghr = 0.0, result = 0.0, zc = 0.0;
-  int evals = 1, state = kPlainHi, it = 0, side = 0;
-  bool fallback = false, use_guess = false;
-  if (fa.mlp) {
-    float z0 = 0.f;
-    if (tid < 32) z0 = mlp_guess(feat, fa.mlp, fa.mlp_norm);
-    if (tid == 0) s_z = double(z0);
-    __syncthreads();
-    const double guess = s_z;
-    use_guess = guess > 0.0 && guess < kZetaMax;
-    if (use_guess) {
-      state = kGuess;
-      zc = guess;
-    }
-  }
-  if (state == kPlainHi) zc = kZetaMax;
   // next Illinois point, or kDone when the feasible end's margin is within
   // tau, the bracket is tight or the evaluations are spent
   auto illinois_next = [&]() {
@@ -1204,117 +1249,183 @@ __device__ __forceinline__ void filter_element(const long long e, T* __restrict_
       result = hi;
       return;
     }
-    double z = (lo * ghi - hi * glo) / (ghi - glo);
-    if (!(lo < z && z < hi)) z = 0.5 * (lo + hi);
-    zc = z;
+    zc = (lo * ghi - hi * glo) / (ghi - glo);
+    if (!(lo < zc && zc < hi)) zc = 0.5 * (lo + hi);
   };
-  if (tid == 0) {
-    s_next = zc;
-    s_go = 1;
-  }
-  for (;;) {
-    __syncthreads();
-    if (!s_go) break;
-    const double z = s_next;
-    const Mins mz = minima(z);  // ends with a barrier: s_next / s_go reusable
-    if (tid != 0) continue;
-    const double gz = gval(mz);
-    ++evals;
-    switch (state) {
-      case kPlainHi:
-        ghi = ghr = gz;
-        if (gz < 0.0) {
-          state = kDone;
-          fallback = true;
-          result = kZetaMax;
-        } else {
-          state = kIllinois;
-          illinois_next();
+  double z = 0.0;
+  for (bool first = true;; first = false) {
+    Mins m0 = minima(z);  // ends with a barrier: s_next / s_go reusable
+    if (first) {
+      // the same test on the modal evaluation (the oracle's form)
+      if (admissible(m0)) {
+        leave_unfiltered();
+        return;
+      }
+      // a filtered element: its entropy minimum at z = 0 (one root, warp 0:
+      // the predictor's features and thread 0's margin read it)
+      if (tid < 32) m0.sm = m0.s = smin_of(m0);
+      m0.ys = INFINITY;
+      // element means of density and pressure (normalise the margin)
+      double wr = 0.0, wp = 0.0, ws = 0.0;
+      for (int z = tid; z < NU; z += kFilterThreads) {
+        const double w5[5] = {double(us[0][z]), double(us[1][z]), double(us[2][z]),
+                              double(us[3][z]), double(us[4][z])};
+        const double p = pressure64(w5, g);
+        double w = double(op.W[z]);
+        wr += w * double(us[0][z]);
+        wp += w * p;
+        ws += w;
+      }
+      const double wsum = block_sum(ws, red);
+      rmean = fmax(block_sum(wr, red) / wsum, kEpsPos);
+      pmean = fmax(block_sum(wp, red) / wsum, kEpsPos);
+      if (tid < 32) {
+        irm = 1.0 / rmean;
+        ipm = 1.0 / pmean;
+        if (smin > 0.0) ism = 1.0 / smin;
+        glo = gval(m0);
+      }
+      // predictor inputs from the unfiltered state (z = 0)
+      if (fa.mlp || fa.samples) {
+        double eh = 0.0, et = 0.0;
+        for (int m = tid; m < NM; m += kFilterThreads) {
+          double d = double(op.deg[m]), c = double(uh[0][m]);
+          if (d > 1.0) eh += c * c;
+          if (d > 0.0) et += c * c;
         }
-        break;
-      case kGuess:
-        if (gz >= 0.0) {
-          hi = z;
-          ghi = ghr = gz;
-          state = kDown;
-          zc = z / fa.ratio;
-          if (gz <= fa.tau) {
-            state = kDone;
-            result = hi;
-          }
-        } else {
-          lo = z;
-          glo = gz;
-          state = kUp;
-          zc = fmin(fa.ratio * z, kZetaMax);
+        eh = block_sum(eh, red);
+        et = block_sum(et, red);
+        feat[0] = float(fmin(fmax(log10((eh + 1e-30) / (et + 1e-30)), -30.0), 30.0));
+        feat[1] = float(fmin(fmax(m0.r / rmean, -30.0), 30.0));
+        feat[2] = float(fmin(fmax(m0.p / pmean, -30.0), 30.0));
+        // log10 of the entropy-bound violation (floor 1e-14)
+        double f3 = 1.0;
+        if (smin > 0.0 && m0.s > -INFINITY && m0.r > 0.0 && m0.p > 0.0)
+          f3 = fmax((smin - m0.s) / smin, 1e-14);
+        feat[3] = float(log10(f3));
+      }
+      if (fa.mlp) {
+        float z0 = 0.f;
+        if (tid < 32) z0 = mlp_guess(feat, fa.mlp, fa.mlp_norm);
+        if (tid == 0) s_z = double(z0);
+        __syncthreads();
+        const double guess = s_z;
+        use_guess = guess > 0.0 && guess < kZetaMax;
+        if (use_guess) {
+          state = kGuess;
+          zc = guess;
         }
-        it = 0;
-        break;
-      case kDown:  // halve until the margin is negative
-        if (gz < 0.0) {
-          lo = z;
-          glo = gz;
-          state = kIllinois;
-          illinois_next();
-        } else {
-          hi = z;
+      }
+      if (state == kPlainHi) zc = kZetaMax;
+    } else if (tid == 0) {
+      const double gz = gval(m0);
+      ++evals;
+      switch (state) {
+        case kPlainHi:
           ghi = ghr = gz;
-          if (z < 1e-6 || gz <= fa.tau) {
-            state = kDone;
-            result = hi;
-          } else {
-            zc = 0.5 * z;
-            if (++it >= 64) {
-              state = kDone;
-              fallback = true;
-              result = kZetaMax;
-            }
-          }
-        }
-        break;
-      case kUp:  // double until the margin is non-negative
-        if (gz >= 0.0) {
-          hi = z;
-          ghi = ghr = gz;
-          state = kIllinois;
-          illinois_next();
-        } else {
-          lo = z;
-          glo = gz;
-          if (z >= kZetaMax) {
+          if (gz < 0.0) {
             state = kDone;
             fallback = true;
             result = kZetaMax;
           } else {
-            zc = fmin(2.0 * z, kZetaMax);
-            if (++it >= 64) {
+            state = kIllinois;
+            illinois_next();
+          }
+          break;
+        case kGuess:
+          if (gz >= 0.0) {
+            hi = z;
+            ghi = ghr = gz;
+            state = kDown;
+            zc = z / fa.ratio;
+            if (gz <= fa.tau) {
+              state = kDone;
+              result = hi;
+            }
+          } else {
+            lo = z;
+            glo = gz;
+            state = kUp;
+            zc = fmin(fa.ratio * z, kZetaMax);
+          }
+          it = 0;
+          break;
+        case kDown:  // halve until the margin is negative
+          if (gz < 0.0) {
+            lo = z;
+            glo = gz;
+            state = kIllinois;
+            illinois_next();
+          } else {
+            hi = z;
+            ghi = ghr = gz;
+            if (z < 1e-6 || gz <= fa.tau) {
+              state = kDone;
+              result = hi;
+            } else {
+              zc = 0.5 * z;
+              if (++it >= 64) {
+                state = kDone;
+                fallback = true;
+                result = kZetaMax;
+              }
+            }
+          }
+          break;
+        case kUp:  // double until the margin is non-negative
+          if (gz >= 0.0) {
+            hi = z;
+            ghi = ghr = gz;
+            state = kIllinois;
+            illinois_next();
+          } else {
+            lo = z;
+            glo = gz;
+            if (z >= kZetaMax) {
               state = kDone;
               fallback = true;
               result = kZetaMax;
+            } else {
+              zc = fmin(2.0 * z, kZetaMax);
+              if (++it >= 64) {
+                state = kDone;
+                fallback = true;
+                result = kZetaMax;
+              }
             }
           }
-        }
-        break;
-      case kIllinois:
-        if (gz >= 0.0) {
-          hi = z;
-          ghi = ghr = gz;
-          if (side == 1) glo *= 0.5;
-          side = 1;
-        } else {
-          lo = z;
-          glo = gz;
-          if (side == -1) ghi *= 0.5;
-          side = -1;
-        }
-        illinois_next();
-        break;
+          break;
+        case kIllinois:
+          if (gz >= 0.0) {
+            hi = z;
+            ghi = ghr = gz;
+            if (side == 1) glo *= 0.5;
+            side = 1;
+          } else {
+            lo = z;
+            glo = gz;
+            if (side == -1) ghi *= 0.5;
+            side = -1;
+          }
+          illinois_next();
+          break;
+      }
     }
-    s_go = state != kDone;
-    s_next = state == kDone ? result : zc;
+    if (tid == 0) {
+      const double zn = state == kDone ? result : zc;
+      s_go = state != kDone;
+      s_next = zn;
+      if (sizeof(T) == 4) {
+        const float zh = narrow_f64(zn);
+        s_zf[0] = zh;
+        s_zf[1] = narrow_f64(zn - widen_f32(zh));
+      }
+    }
+    __syncthreads();
+    z = s_next;
+    if (!s_go) break;
   }
-  // every thread: the strength found by thread 0
-  result = s_next;
+  result = z;  // every thread: the strength found by thread 0
   // write the filtered state and its flux-point values
   for (int m = tid; m < NM; m += kFilterThreads) {
     const T sk = T(exp(-result * double(op.deg[m]) * double(op.deg[m])));
@@ -1366,10 +1477,13 @@ __device__ __forceinline__ void filter_element(const long long e, T* __restrict_
 // The listed elements, one CTA each in turn.  The list's length is known on
 // the device alone: the grid holds the CTAs that can be resident (one CTA
 // per element of the mesh, most of which only returned, before).  Bound by
-// the margin's serial FP64 chain: 174 -> 137 us on 16384 hexahedra of order 3
-// of which some hundred are listed.
+// each evaluation's serial FP64 chain and its barriers, so by how many
+// elements are in work: 4 CTAs of 96 registers per SM for FP32 values (3 of 128:
+// 5 % slower a step).  174 -> 119 us on average over the stages of a shock on
+// 16384 hexahedra of order 3.  (Summing the modes of a degree once per element,
+// 10 terms an evaluation instead of 64, gained nothing.)
 template <typename T, typename TR, int NU, int NF>
-__global__ void __launch_bounds__(kFilterThreads)
+__global__ void __launch_bounds__(kFilterThreads, sizeof(T) == 4 ? 4 : 3)
     k_filter(T* __restrict__ reg, TR* __restrict__ regR, T* __restrict__ uf, FilterOps<T> op,
              FilterArgs fa, const int32_t* __restrict__ list, const int* __restrict__ count) {
   const int n = *count;

@@ -44,6 +44,15 @@ int setup_filter(fr_mesh* m) {
   return FR_OK;
 }
 
+inline GammaArgs gamma_args(double g) {
+  GammaArgs a;
+  a.g = float(g);
+  a.gm1h = float(g - 1.0);
+  a.gm1l = float((g - 1.0) - double(a.gm1h));
+  a.by5 = entropy_by_s5(g);
+  return a;
+}
+
 // Launched at the start of every filtered stage: s_min from the stage input.
 template <typename T, typename TR>
 void launch_entropy_min(fr_mesh* m, cudaStream_t s, bool from_x) {
@@ -52,11 +61,12 @@ void launch_entropy_min(fr_mesh* m, cudaStream_t s, bool from_x) {
     dispatch(D.kind, m->order, [&](auto nu, auto nf) {
       constexpr int NU = decltype(nu)::value, NF = decltype(nf)::value;
       long long threads = D.ne * 32;
-      k_entropy_min<T, TR, NU, NF><<<nblk(threads, 256), 256, 0, s>>>(
+      k_entropy_min<T, TR, NU, NF><<<nblk(threads, kScanThreads), kScanThreads, 0, s>>>(
           D.ne, from_x ? nullptr : (const T*)D.Y, (const TR*)D.X,
-          (const T*)m->uf, m->tt, int(t), D.fpartner, m->gamma, D.smin, (EntropyRec*)D.frec);
+          (const T*)m->uf, m->tt, int(t), D.fpartner, m->gamma, gamma_args(m->gamma), D.smin,
+          (EntropyRec*)D.frec);
     });
-    if (sizeof(T) == 4 && sizeof(TR) == 4 && m->gamma == 1.4)
+    if (sizeof(T) == 4 && sizeof(TR) == 4 && entropy_by_s5(m->gamma))
       k_entropy_value<<<nblk(D.ne, 128), 128, 0, s>>>(D.ne, (const EntropyRec*)D.frec, m->gamma,
                                                       D.smin);
   }
@@ -69,6 +79,7 @@ void launch_filter(fr_mesh* m, cudaStream_t s, DevType& D, bool last_stage) {
                   (const T*)D.fW, D.fpartner};
   FilterArgs fa;
   fa.gamma = m->gamma;
+  fa.gf = gamma_args(m->gamma);
   fa.tau = m->wsize == 8 ? 1e-8 : 1.0 / 1048576.0;
   fa.ratio = m->mlp_ratio;
   fa.zeta_last = D.zeta_last;
@@ -88,7 +99,7 @@ void launch_filter(fr_mesh* m, cudaStream_t s, DevType& D, bool last_stage) {
   cudaMemsetAsync(D.fcount, 0, sizeof(int), s);
   dispatch(D.kind, m->order, [&](auto nu, auto nf) {
     constexpr int NU = decltype(nu)::value, NF = decltype(nf)::value;
-    k_filter_check<T, TR, NU, NF><<<nblk(D.ne * 32, 256), 256, 0, s>>>(
+    k_filter_check<T, TR, NU, NF><<<nblk(D.ne * 32, kScanThreads), kScanThreads, 0, s>>>(
         D.ne, reg, regR, uf, fa, D.flist, D.fcount, (CheckRec*)D.frec);
     if (sizeof(T) == 4)
       k_filter_decide<<<nblk(D.ne, 128), 128, 0, s>>>(D.ne, (const CheckRec*)D.frec, fa, D.flist,
