@@ -140,23 +140,27 @@ def kernel_models(nu, nf, ne, w, wr, npair):
     w: bytes of a trace/stage value, wr: bytes of a solution register."""
     n = round(nu ** (1.0 / 3.0))
     # FP64 values: 15 gradient components per flux point go to the face
-    # kernel; FP32 values: 5 viscous normal-flux values q per flux point
-    # (plus the 5 solution traces the grad kernel reads to form q)
-    gf = 15 if w == 8 else 10
+    # kernel; FP32 values: 4 viscous normal-flux values q per flux point (the
+    # mass component stays zero), with the 3 normal components they need
+    gf = 15 if w == 8 else 7
     bytes_ = {
-        # u(5) + metrics(10) + du(5 per flux pt) in, grad(15) + gradf out
-        "grad": ne * (w * (5 * nu + 10 * nu + 5 * nf + 15 * nu + gf * nf)),
-        # u(5) + grad(15) + metrics(10) + F^C(5/fpt) in; Y and u_f out;
-        # solution register X in and out
-        "volume": ne * (w * (5 * nu + 15 * nu + 10 * nu + 5 * nf + 5 * nu
+        # u(5) + metrics(10) + both traces (10 per flux pt) and the partner
+        # codes in, viscous flux(9) + gradf out
+        "grad": ne * (w * (5 * nu + 10 * nu + 9 * nu + 10 * nf + gf * nf) + 4 * nf),
+        # u(5) + viscous flux(9) + metrics(10) + F^C(5/fpt) in; Y and u_f
+        # out; solution register X in and out
+        "volume": ne * (w * (5 * nu + 9 * nu + 10 * nu + 5 * nf + 5 * nu
                              + 5 * nf) + wr * 10 * nu),
         "face_ucommon": npair * (w * 20 + 8),
         "face_flux": npair * (w * (2 * (20 if w == 8 else 10) + 5 + 10) + 8),
     }
+    # FP64: the line operators and metric products are sums on the integer
+    # pipe; the pointwise physics counts against the FP64 rate
     flops = {
-        "grad": ne * (2 * nu * (15 * n + 30 + 45) + 15 * nu
-                      + 2 * nf * 15 * n),
-        "volume": ne * (nu * (30 + 150 + 90 + 2 * 5 * (3 * n + 6) + 25)
+        "grad": ne * (nu * 110 if w == 8 else
+                      2 * nu * (15 * n + 30 + 45) + 15 * nu + nu * 75 + 2 * nf * 15 * n),
+        "volume": ne * (nu * 75 if w == 8 else
+                        nu * (75 + 90 + 2 * 5 * (3 * n + 6) + 25)
                         + 2 * nf * 5 * n + 5 * nf + 2 * nf * 5 * n),
         "face_ucommon": npair * 10,
         "face_flux": npair * 330,

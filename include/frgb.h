@@ -261,7 +261,8 @@ int fr_rk_adaptive_step(fr_mesh* mesh, fr_adapt_t* ctl, double* dt, int* accepte
  * CUDA events around every launch on the handle's stream.  On return
  * ms[k] holds the summed device time (milliseconds) and launches[k] the
  * launch count of kernel class k during that step, for k < FR_KC_COUNT. */
-enum { FR_KC_FACE_U = 0,  /* NS common solution at interior flux points */
+enum { FR_KC_FACE_U = 0,  /* NS common solution at interior flux points (only
+                           * where the gradient kernels do not form it) */
        FR_KC_BND_U = 1,   /* NS common solution at boundary flux points */
        FR_KC_GRAD = 2,    /* NS corrected gradients (one launch per type) */
        FR_KC_FACE_F = 3,  /* common normal flux, interior pairs */
@@ -330,9 +331,9 @@ int fr_get_tuning(const fr_mesh* mesh, int* active, float* ms_per_step);
  * kept; "Task graphs": independent kernels run in parallel).  Indexed by
  * element kind (FR_HEX8, FR_PRI6, FR_TET4):
  *   tile_grad, tile_vol: gradient / volume kernel tile: elements per CTA of
- *     the sum-factorised hexahedron kernels (at most 256 threads per CTA),
- *     persistent CTAs per SM of the dense kernels; 0 = the largest (default),
- *     -1 = no such element in the mesh;
+ *     the sum-factorised hexahedron kernels (at most 288 threads per CTA),
+ *     persistent CTAs per SM of the prism and tetrahedron kernels; 0 = the
+ *     largest (default), -1 = no such element in the mesh;
  *   tensor_grad, tensor_vol: 1 when that kernel runs on the tensor cores;
  *   structured: 1 when the CUDA-core kernels of that kind use the
  *     structure of its operators (Section 3.1, "Matrix multiplications":
