@@ -23,8 +23,9 @@
 // As on hexahedra the gradient kernel stores the viscous flux at the solution
 // points (9 values) in place of the gradient (15).
 //
-// Bound by latency between the phases' barriers (DRAM traffic would take
-// about half the time).  Measured, us: common solution + gradient, volume
+// Bound by the shared-memory pipe (66-82 % of its rate at p = 3) and the
+// barriers between the phases; DRAM traffic would take a third to a half of the
+// time (27-35 %).  Measured, us: common solution + gradient, volume
 // with one thread per point -> here, the gradient with its jumps:
 //   384000 tetrahedra p = 1    59 + 195, 181 -> 127,  86
 //   196608 tetrahedra p = 2    50 + 200, 256 -> 148, 124
