@@ -1,18 +1,16 @@
-// FP64 hexahedron kernels whose linear operators run on the integer pipe.
+// FP64 hexahedron kernels whose line operators run on the integer pipe.
 //
 // GB300 issues FP64 instructions at 2 lanes per clock and SM, and 32 x 32 +
 // 64-bit integer multiply-adds (IMAD.WIDE) at 64 (measured: 54.6 against 1.6
-// per clock in chains of each).  The FP64 gradient and volume kernels were
-// bound by that FP64 pipe (0.94 of its rate), most of it in products with
-// the line operators and the metric.  Here those products are fixed-point
-// sums:
+// per clock in chains of each).  FP64 gradient and volume kernels are bound by
+// that FP64 pipe, most of it in products with the line operators.  Here those
+// products are fixed-point sums:
 //
-//   - a field (one variable of one element) is converted to fixed point
-//     relative to its largest magnitude in the element, q = v 2^(59 - E),
-//     |v| < 2^E, held as two signed limbs q = hi 2^30 + lo (8 bytes, as the
-//     double it replaces);
-//   - operator and metric entries are limbs too, scaled by a power of two
-//     that bounds the row's sum of magnitudes, so no sum can overflow;
+//   - the N points of a line, and the values at its two faces, are converted
+//     to fixed point relative to the largest magnitude among them,
+//     q = v 2^(59 - E), |v| < 2^E, held as two signed limbs q = hi 2^30 + lo;
+//   - operator entries are limbs too, scaled by a power of two that bounds the
+//     row's sum of magnitudes, so no sum can overflow;
 //   - a term is three multiply-adds, hi hi' into one 64-bit sum and
 //     hi lo' + lo hi' into another (lo lo' is below the result's unit);
 //   - the derivative and interpolation rows of the symmetric line points
@@ -21,28 +19,30 @@
 //   - a result has a unit of about 2^-60 of its bound |A|_inf max|v| and is
 //     normalised and rounded once to FP64.
 //
-// FP64 multiply-adds round every partial sum.  Over random smooth fields and
-// sheared metrics the chain flux -> transformed flux -> jump -> divergence at a
-// point is 4e-16, 1.1e-15 and 1.0e-15 (rms, p = 2, 3, 4, for a flux of one)
-// from exact rational arithmetic with the exact operators; FP64 loops with
-// FP64 operators are 1.3e-14, 4e-15 and 1.1e-13 from it.  The flux, the
-// scaling by 1/J and the RK update stay in FP64.  A field that holds an Inf
-// or NaN gives NaN, which the epilogue flags as before.
+// The unit belongs to the line and the variable: an FP64 sum over the same
+// line rounds its partial sums to 2^-53 of those magnitudes, whatever the
+// other lines, directions and variables of the element hold.  (One exponent
+// per element and field, and metric products in fixed point, lost as many bits as
+// an element is stretched or a field varies within it.)  Metric products, the
+// flux, the scaling by 1/J and the RK update stay in FP64; the divergence's
+// three directions are added in units of the largest.  A line that holds an Inf
+// or NaN gives NaN, which the epilogue flags.
 //
-// Threads: TPE = 32 ceil(N^3 / 32) per element (whole warps, so that the
-// field maxima reduce by warp), one per solution point in the pointwise
-// phases and one per (field, line) in the line phases.  A line thread reads
-// its N points once for all N results (and both face values), with
+// Threads: TPE = 32 ceil(N^3 / 32) per element, one per solution point in the
+// pointwise phases and one per (field, line) in the line phases.  A line thread
+// reads its N points once for all N results (and both face values), with
 // coefficients that are the same for every thread (constant operands);
-// one thread per point read every line N times, with lane-varying
+// one thread per point would read every line N times, with lane-varying
 // coefficients.
 //
-// Measured per launch, 24^3 p = 4 (20^3 p = 3) Navier-Stokes: gradient 850 -> 301
-// us (242 -> 100; 344 with the solution jumps taken in the kernel, which
-// saves the 43 us of a kernel for them), volume 1108 -> 268 us (321 -> 95).  What bounds them now:
-// the ALU pipe and the FP64 pipe are each at 48-59 %, the rest is the latency
-// of dependent integer instructions at 24 warps per SM (80 registers; 64
-// spill, 96 leave fewer warps, both slower).
+// Measured per launch, 24^3 p = 4 (20^3 p = 3) Navier-Stokes: gradient with the
+// solution jumps 850 + 43 -> 427 us (242 + 20 -> 140), volume 1108 -> 292 us
+// (321 -> 94), against FP64 loops with one thread per point; one exponent per
+// element and field and metric products in fixed point took 345 and 269 us
+// (118, 96).  The gradient kernel is bound by the FP64 pipe, some 110
+// instructions a point of 64 clocks a warp; the volume kernel has 90 of them
+// and as much time in integer instructions.  62 to 70 registers; a fourth CTA
+// per SM gained nothing.
 #pragma once
 #include "fr_hex.cuh"
 
@@ -98,27 +98,21 @@ __device__ __forceinline__ long long fx_join(FxCoef a) {
   return (long long)a.hi * (1 << 30) + a.lo;
 }
 
-// a 64-bit integer as the two words of a slot
-__device__ __forceinline__ FxCoef fx_pack(long long q) {
-  return FxCoef{int(q >> 32), int(uint32_t(q))};
-}
-
-__device__ __forceinline__ long long fx_unpack(FxCoef a) {
-  return (long long)(((unsigned long long)uint32_t(a.hi) << 32) | uint32_t(a.lo));
-}
-
-// magnitude bits of v's high word: the field maximum reduces on these
+// magnitude bits of v's high word: the largest of a line sets its exponent
 __device__ __forceinline__ unsigned fx_mag(double v) {
   return unsigned(__double2hiint(v)) & 0x7fffffffu;
 }
 
-// Field exponents below this are taken as this (values under 2^-890 resolve
+// Line exponents below this are taken as this (values under 2^-890 resolve
 // to 2^-949): the shifts below then need no special case for zero.
 constexpr int kFxMinExp = 132;
 
-// v 2^(59 - E) for the field exponent em = E + 1022 (the biased exponent
-// field of the largest magnitude, or more), truncated
-__device__ __forceinline__ long long fx_from(double v, int em) {
+// exponent em = E + 1022 of a line whose largest magnitude has the bits mag:
+// the biased exponent field, or more
+__device__ __forceinline__ int fx_exp(unsigned mag) { return max(int(mag >> 20), kFxMinExp); }
+
+// v 2^(59 - E), truncated toward zero (odd in v)
+__device__ __forceinline__ FxCoef fx_limbs(double v, int em) {
   const int h = __double2hiint(v), s = h >> 31;
   const unsigned l = unsigned(__double2loint(v));
   const unsigned mh = (unsigned(h) & 0xfffffu) | 0x100000u;
@@ -126,19 +120,20 @@ __device__ __forceinline__ long long fx_from(double v, int em) {
       ((unsigned long long)__funnelshift_l(l, mh, 6) << 32) | (l << 6);
   unsigned long long q;  // a shift by 64 or more gives 0
   asm("shr.b64 %0, %1, %2;" : "=l"(q) : "l"(m), "r"(em - ((h >> 20) & 0x7ff)));
-  // (the sign as one's complement: one unit)
-  return (long long)(q ^ (((unsigned long long)unsigned(s) << 32) | unsigned(s)));
+  const FxCoef a = fx_split((long long)q);
+  return FxCoef{(a.hi ^ s) - s, (a.lo ^ s) - s};
 }
 
-// Whether every result of a field with exponent em (and a metric exponent
-// jx) is a normal number; a field with Inf / NaN (em = 2047) is not.
-__device__ __forceinline__ bool fx_edge(int em, int jx = 1023) {
-  return em < 300 || em > 1800 || jx < 700 || jx > 1400;
+// Lines whose results need the general conversion: one with an Inf or NaN
+// (exponent 2047), or with magnitudes outside 2^[-722, 777] that do not all
+// vanish.
+__device__ __forceinline__ bool fx_edge(unsigned mag) {
+  return mag != 0 && (mag >> 20) - 300u > 1500u;
 }
 
-// R 2^(bx - 1023) for a field that fx_edge names
-static __device__ __noinline__ double fx_to_edge(long long R, int bx, bool bad) {
-  if (bad) return __longlong_as_double(0x7ff8000000000000LL);
+// R 2^(bx - 1023) for a line that fx_edge names
+static __device__ __noinline__ double fx_to_edge(long long R, int bx, unsigned mag) {
+  if (mag >= 0x7ff00000u) return __longlong_as_double(0x7ff8000000000000LL);
   return ldexp(double(R), bx - 1023);
 }
 
@@ -176,14 +171,14 @@ template <int N>
 struct FxPairs {
   static constexpr int P = N / 2, H = (N + 1) / 2;
   FxCoef e[H], o[P > 0 ? P : 1];
-  __device__ __forceinline__ void load(const FxCoef* p, int st) {
+  __device__ __forceinline__ void set(const double (&v)[N], int em) {
 #pragma unroll
     for (int m = 0; m < P; ++m) {
-      const FxCoef x = p[m * st], y = p[(N - 1 - m) * st];
+      const FxCoef x = fx_limbs(v[m], em), y = fx_limbs(v[N - 1 - m], em);
       e[m] = FxCoef{x.hi + y.hi, x.lo + y.lo};
       o[m] = FxCoef{x.hi - y.hi, x.lo - y.lo};
     }
-    if (N % 2) e[P] = p[P * st];
+    if (N % 2) e[P] = fx_limbs(v[P], em);
   }
   // values at the two faces in units of the interpolation row
   __device__ __forceinline__ void faces(const HexFxOps& op, long long* f0, long long* f1) const {
@@ -243,37 +238,35 @@ __device__ __forceinline__ void fx_sync(int le) {
   }
 }
 
-// Maxima over an element of NV magnitudes per thread: warp maxima to
-// ex[warp][NV], read after the caller's fx_sync by fx_field_max.
-template <int NV>
-__device__ __forceinline__ void fx_warp_max(const unsigned (&m)[NV], unsigned* ex, int w) {
+// the N values of a line and their largest magnitude (joined to mag)
+template <int N>
+__device__ __forceinline__ unsigned fx_load(const double* p, int st, double (&v)[N],
+                                            unsigned mag = 0) {
 #pragma unroll
-  for (int k = 0; k < NV; ++k) {
-    const unsigned r = __reduce_max_sync(0xffffffffu, m[k]);
-    if ((threadIdx.x & 31) == 0) ex[w * NV + k] = r;
+  for (int m = 0; m < N; ++m) {
+    v[m] = p[m * st];
+    mag = max(mag, fx_mag(v[m]));
   }
+  return mag;
 }
 
-template <int NV, int WPE>
-__device__ __forceinline__ unsigned fx_field_max(const unsigned* ex, int k) {
-  unsigned r = ex[k];
-#pragma unroll
-  for (int w = 1; w < WPE; ++w) r = max(r, ex[w * NV + k]);
-  return r;
-}
-
-// The same into words that are zero before (an earlier barrier): lane q
-// of each warp adds the warp's maximum of field q.
-template <int NV>
-__device__ __forceinline__ void fx_max_to(const unsigned (&m)[NV], unsigned* ex) {
-  const unsigned lane = threadIdx.x & 31;
-  unsigned mine = 0;
-#pragma unroll
-  for (int k = 0; k < NV; ++k) {
-    const unsigned r = __reduce_max_sync(0xffffffffu, m[k]);
-    if (lane == k) mine = r;
+// values at a line's two faces
+template <int N>
+__device__ __forceinline__ void fx_faces(const HexFxOps& op, const double* p, int st, double* f0,
+                                         double* f1) {
+  double v[N];
+  const unsigned mag = fx_load<N>(p, st, v);
+  const int em = fx_exp(mag), bx = em - 1022 + op.sm - 59 + 1023;
+  FxPairs<N> w;
+  long long r0, r1;
+  w.set(v, em);
+  w.faces(op, &r0, &r1);
+  *f0 = fx_to(r0, bx);
+  *f1 = fx_to(r1, bx);
+  if (fx_edge(mag)) {
+    *f0 = fx_to_edge(r0, bx, mag);
+    *f1 = fx_to_edge(r1, bx, mag);
   }
-  if (lane < NV) atomicMax(ex + lane, mine);
 }
 
 // line l of direction d: first slot and stride in a field, and the flux
@@ -287,198 +280,103 @@ __device__ __forceinline__ void fx_line(int d, int l, int* s0, int* st, int* fm)
   *fm = 2 * d * G::N2 + l;
 }
 
-// Fixed-point metric of an element: S (one exponent) and, for Navier-Stokes,
-// S / det J (one exponent per physical direction, the columns of S).  ex
-// [ne][4]: exponents em (as fx_from) of S and of the three columns.  One
-// warp per element; built once per mesh.
-template <int NU>
-__global__ void k_fx_metric(long long ne, const double* __restrict__ smat,
-                            const double* __restrict__ rcpdjac, FxCoef* __restrict__ sq,
-                            FxCoef* __restrict__ jq, int* __restrict__ ex) {
-  const int lane = threadIdx.x & 31;
-  const long long e = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (e >= ne) return;  // whole warps
-  unsigned m[4] = {0, 0, 0, 0};
-  for (int z = lane; z < NU; z += 32)
-    for (int r = 0; r < 9; ++r) {
-      const double s = smat[(e * 9 + r) * NU + z];
-      m[0] = max(m[0], fx_mag(s));
-      m[1 + r % 3] = max(m[1 + r % 3], fx_mag(s * rcpdjac[e * NU + z]));
-    }
-  for (int k = 0; k < 4; ++k) {
-    m[k] = max(__reduce_max_sync(0xffffffffu, m[k]) >> 20, unsigned(kFxMinExp));
-    if (lane == 0) ex[e * 4 + k] = int(m[k]);
-  }
-  // limbs below 2^58: one bit less than a field's, for sums of three
-  for (int z = lane; z < NU; z += 32)
-    for (int r = 0; r < 9; ++r) {
-      const long long i = (e * 9 + r) * NU + z;
-      const double s = smat[i];
-      sq[i] = fx_split(fx_from(s, int(m[0]) + 1));
-      if (jq) jq[i] = fx_split(fx_from(s * rcpdjac[e * NU + z], int(m[1 + r % 3]) + 1));
-    }
-}
-
-// Shared memory per element (8-byte slots): gradient u [5][PN], du [5][NF],
-// gradient [15][PN]; volume f~ [15][PN], F^C / jump [5][NF]; then warp maxima
-// of up to 6 fields, element maxima of up to 15 and 8 exponents.
+// Shared memory per element: gradient u [5][PN], du [5][NF], gradient [15][PN];
+// volume F^C [5][NF], f~ [15][PN] (8-byte slots), line magnitudes [15][N2].
 template <int N>
 __host__ __device__ constexpr int hexfx_bytes_per_elem(bool grad) {
   using G = FxGeom<N>;
-  const int slots = (grad ? 20 : 15) * G::PN + 5 * G::NF;
-  return (slots * 8 + (G::WPE * 6 + 16 + 8) * 4 + 15) / 16 * 16;
+  return ((grad ? 20 : 15) * G::PN * 8 + 5 * G::NF * 8 + (grad ? 0 : 15 * G::N2 * 4) + 15) / 16 *
+         16;
 }
 
-// NS gradients: corrected reference gradient
-// by lines, physical gradient by the fixed-point S / det J, its 15 components
-// at the flux points by lines.  At the solution points the volume kernel
-// needs the viscous flux alone: it is formed here, where the FP64 pipe is
-// otherwise idle, and stored as stress and energy flux [ne][9][nu] (15
-// gradient components would also be 6 more to write and read).  RAW: the
-// gradient itself [ne][15][nu], for the anti-aliased flux.
+// NS gradients: corrected reference gradient by lines, physical gradient by
+// S / det J, its 15 components at the flux points by lines.  At the solution
+// points the volume kernel needs the viscous flux alone: stored as stress and
+// energy flux [ne][9][nu] (15 gradient components would also be 6 more to
+// write and read).  RAW: the gradient itself [ne][15][nu], for the
+// anti-aliased flux.
 template <int N, int EPB, bool RAW>
 __global__ void __launch_bounds__(EPB* FxGeom<N>::TPE, N == 3 ? 2 : 3)
     k_hexfx_grad(long long ne, const double* __restrict__ u,
-                 const __grid_constant__ TraceArgs<double> ta,
-                 const FxCoef* __restrict__ jq, const int* __restrict__ jex,
-                 const __grid_constant__ HexFxOps op, Phys<double> ph,
-                 double* __restrict__ grad, double* __restrict__ gradf) {
+                 const __grid_constant__ TraceArgs<double> ta, const double* __restrict__ smat,
+                 const double* __restrict__ rcpdjac, const __grid_constant__ HexFxOps op,
+                 Phys<double> ph, double* __restrict__ grad, double* __restrict__ gradf) {
   using G = FxGeom<N>;
   constexpr int NU = G::NU, NF = G::NF, N2 = G::N2, TPE = G::TPE, PN = G::PN;
   constexpr int NFT = (NF + TPE - 1) / TPE;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int le = threadIdx.x / TPE, z = threadIdx.x - le * TPE, wz = z >> 5;
+  const int le = threadIdx.x / TPE, z = threadIdx.x - le * TPE;
   const long long e = (long long)blockIdx.x * (blockDim.x / TPE) + le;
   if (e >= ne) return;  // whole elements: their barriers are their own
-  FxCoef* us = reinterpret_cast<FxCoef*>(smem_raw + le * hexfx_bytes_per_elem<N>(true));
-  FxCoef* ds = us + 5 * PN;
-  FxCoef* gs = ds + 5 * NF;  // [15][PN]: integers by fx_pack, then limbs
-  unsigned* ex = reinterpret_cast<unsigned*>(gs + 15 * PN);
-  unsigned* eg = ex + 6 * G::WPE;                  // [15] gradient maxima
-  int* ek = reinterpret_cast<int*>(eg + 16);       // [5] fields, [3] metric
+  double* us = reinterpret_cast<double*>(smem_raw + le * hexfx_bytes_per_elem<N>(true));
+  double* ds = us + 5 * PN;
+  double* gs = ds + 5 * NF;
   const bool pt = z < NU;
-  const int a = z % N, b = (z / N) % N, c = z / N2;
-  const int slot = G::slot(a, b, c);
-  if (z < 15) eg[z] = 0;
-  int em[5];
-  {
-    double uv[5], dv[NFT][5];
-    unsigned mx[5];
+  const int slot = G::slot(z % N, (z / N) % N, z / N2);
 #pragma unroll
-    for (int k = 0; k < 5; ++k) {
-      uv[k] = pt ? u[(e * 5 + k) * NU + z] : 0.0;
-      mx[k] = fx_mag(uv[k]);
-    }
+  for (int i = 0; i < NFT; ++i) {
+    if (z + i * TPE < NF) {
+      double own[5], dv[5];
+      trace_jump(ta, e, z + i * TPE, NF, own, dv);
 #pragma unroll
-    for (int i = 0; i < NFT; ++i) {
-      if (z + i * TPE < NF) {
-        double own[5];
-        trace_jump(ta, e, z + i * TPE, NF, own, dv[i]);
-#pragma unroll
-        for (int k = 0; k < 5; ++k) mx[k] = max(mx[k], fx_mag(dv[i][k]));
-      }
-    }
-    fx_warp_max<5>(mx, ex, wz);
-    fx_sync<G::WPE, EPB>(le);
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-      em[k] = max(int(fx_field_max<5, G::WPE>(ex, k) >> 20), kFxMinExp);
-      if (pt) us[k * PN + slot] = fx_split(fx_from(uv[k], em[k]));
-#pragma unroll
-      for (int i = 0; i < NFT; ++i)
-        if (z + i * TPE < NF) ds[k * NF + z + i * TPE] = fx_split(fx_from(dv[i][k], em[k]));
+      for (int k = 0; k < 5; ++k) ds[k * NF + z + i * TPE] = dv[k];
     }
   }
+  if (pt) {
+#pragma unroll
+    for (int k = 0; k < 5; ++k) us[k * PN + slot] = u[(e * 5 + k) * NU + z];
+  }
   fx_sync<G::WPE, EPB>(le);
-  // lines: (variable, direction, line) -> N reference-gradient values in
-  // units of 2^(E + sg - 60)
+  // lines: (variable, direction, line) -> N reference-gradient values
   for (int t = z; t < 15 * N2; t += TPE) {
     const int k = t / (3 * N2), r = t - k * 3 * N2, d = r / N2, l = r - d * N2;
     int s0, st, fm;
     fx_line<N>(d, l, &s0, &st, &fm);
-    FxPairs<N> v;
-    v.load(us + k * PN + s0, st);
+    const double j0 = ds[k * NF + fm], j1 = ds[k * NF + fm + N2];
+    double v[N];
+    const unsigned mag = fx_load<N>(us + k * PN + s0, st, v, max(fx_mag(j0), fx_mag(j1)));
+    const int em = fx_exp(mag), bx = em - 1022 + op.sg - 60 + 1023;
+    FxPairs<N> w;
+    w.set(v, em);
     long long o[N];
-    v.template derivative<1>(op.g, ds[k * NF + fm], ds[k * NF + fm + N2], o);
+    w.template derivative<1>(op.g, fx_limbs(j0, em), fx_limbs(j1, em), o);
+    double* q = gs + (d * 5 + k) * PN + s0;
 #pragma unroll
-    for (int i = 0; i < N; ++i) gs[(d * 5 + k) * PN + s0 + i * st] = fx_pack(o[i]);
+    for (int i = 0; i < N; ++i) q[i * st] = fx_to(o[i], bx);
+    if (fx_edge(mag)) {
+#pragma unroll
+      for (int i = 0; i < N; ++i) q[i * st] = fx_to_edge(o[i], bx, mag);
+    }
   }
-  FxCoef J[9];
-  int jx[3];
+  double S[9], rj = 0.0;
   if (pt) {
 #pragma unroll
-    for (int r = 0; r < 9; ++r) J[r] = jq[(e * 9 + r) * NU + z];
-  }
-#pragma unroll
-  for (int j = 0; j < 3; ++j) jx[j] = jex[e * 4 + 1 + j];
-  bool edge = false;
-#pragma unroll
-  for (int k = 0; k < 5; ++k) edge |= fx_edge(em[k], jx[k % 3]);
-  if (z == 0) {
-#pragma unroll
-    for (int k = 0; k < 5; ++k) ek[k] = em[k];
-#pragma unroll
-    for (int j = 0; j < 3; ++j) ek[5 + j] = jx[j];
+    for (int r = 0; r < 9; ++r) S[r] = smat[(e * 9 + r) * NU + z];
+    rj = rcpdjac[e * NU + z];
   }
   fx_sync<G::WPE, EPB>(le);
-  // physical gradient g[j][k] = sum_i (S_ij / det J) gref_i, in units of
-  // 2^(E + sg + E_j - 61), in place of the reference gradient of the point
-  const int b0 = op.sg - 1022 - 1022 - 61 + 1023;  // + em + jx: exponent of a unit
-  double g[3][5];
-  unsigned mg[15];
-#pragma unroll
-  for (int q = 0; q < 15; ++q) mg[q] = 0;
   if (pt) {
+#pragma unroll
+    for (int r = 0; r < 9; ++r) S[r] *= rj;
+    double g[3][5];
+    double* p = gs + slot;
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
-      FxCoef r[3];
-#pragma unroll
-      for (int i = 0; i < 3; ++i) r[i] = fx_split(fx_unpack(gs[(i * 5 + k) * PN + slot]));
+      const double g0 = p[k * PN], g1 = p[(5 + k) * PN], g2 = p[(10 + k) * PN];
 #pragma unroll
       for (int j = 0; j < 3; ++j) {
-        FxSum<3> s;
-#pragma unroll
-        for (int i = 0; i < 3; ++i) s.add(J[i * 3 + j], r[i]);
-        const long long x = s.value();
-        const int h = int(x >> 32);
-        mg[j * 5 + k] = unsigned(h ^ (h >> 31));
-        gs[(j * 5 + k) * PN + slot] = fx_pack(x);
-        g[j][k] = fx_to(x, b0 + em[k] + jx[j]);
+        g[j][k] = S[j] * g0 + S[3 + j] * g1 + S[6 + j] * g2;
+        p[(j * 5 + k) * PN] = g[j][k];
+        if (RAW) grad[(e * 15 + j * 5 + k) * NU + z] = g[j][k];
       }
     }
-    if (edge) {
-#pragma unroll
-      for (int j = 0; j < 3; ++j)
-#pragma unroll
-        for (int k = 0; k < 5; ++k)
-          g[j][k] = fx_to_edge(fx_unpack(gs[(j * 5 + k) * PN + slot]), b0 + em[k] + jx[j],
-                               em[k] >= 2047);
-    }
-  }
-  fx_max_to<15>(mg, eg);
-  if (pt) {
-    if (RAW) {
-#pragma unroll
-      for (int j = 0; j < 3; ++j)
-#pragma unroll
-        for (int k = 0; k < 5; ++k) grad[(e * 15 + j * 5 + k) * NU + z] = g[j][k];
-    } else {
+    if (!RAW) {
       double uz[5], tq[9];
 #pragma unroll
-      for (int k = 0; k < 5; ++k) uz[k] = u[(e * 5 + k) * NU + z];
+      for (int k = 0; k < 5; ++k) uz[k] = us[k * PN + slot];
       viscous_point(uz, g, ph, tq);
 #pragma unroll
       for (int r = 0; r < 9; ++r) grad[(e * 9 + r) * NU + z] = tq[r];
-    }
-  }
-  fx_sync<G::WPE, EPB>(le);
-  // each component shifted to the full width of its largest value, |x| < 2^(64
-  // - clz): to below 2^63, then 2^59
-  if (pt) {
-#pragma unroll
-    for (int q = 0; q < 15; ++q) {
-      const int sh = __clz(int(eg[q])) - 1;
-      gs[q * PN + slot] = fx_split((fx_unpack(gs[q * PN + slot]) << sh) >> 4);
     }
   }
   fx_sync<G::WPE, EPB>(le);
@@ -488,175 +386,91 @@ __global__ void __launch_bounds__(EPB* FxGeom<N>::TPE, N == 3 ? 2 : 3)
     const int k = t / (3 * N2), r = t - k * 3 * N2, d = r / N2, l = r - d * N2;
     int s0, st, fm;
     fx_line<N>(d, l, &s0, &st, &fm);
-    const int bk = b0 + ek[k] + op.sm + 5;
-    long long f[6];
-    double v[6];
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      FxPairs<N> w;
-      w.load(gs + (j * 5 + k) * PN + s0, st);
-      w.faces(op, f + 2 * j, f + 2 * j + 1);
-    }
-    int bx[3];
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      bx[j] = bk + ek[5 + j] - __clz(int(eg[j * 5 + k]));
-      v[2 * j] = fx_to(f[2 * j], bx[j]);
-      v[2 * j + 1] = fx_to(f[2 * j + 1], bx[j]);
-    }
-    if (edge) {
-#pragma unroll
-      for (int i = 0; i < 6; ++i) v[i] = fx_to_edge(f[i], bx[i / 2], ek[k] >= 2047);
-    }
     double* o = gradf + (e * 15 + k) * NF + fm;
 #pragma unroll
-    for (int i = 0; i < 6; ++i) o[(i / 2) * 5 * NF + (i % 2) * N2] = v[i];
+    for (int j = 0; j < 3; ++j) {
+      double f0, f1;
+      fx_faces<N>(op, gs + (j * 5 + k) * PN + s0, st, &f0, &f1);
+      o[j * 5 * NF] = f0;
+      o[j * 5 * NF + N2] = f1;
+    }
   }
 }
 
-// Volume kernel: flux in FP64, f~ = S F, jump, divergence and
-// correction in fixed point, R = -div / J and the RK epilogue in FP64, the
-// next stage's u_f by lines in fixed point.  The three momentum variables
-// share one field exponent (their flux tensor is symmetric).  visc: the
-// viscous flux of k_hexfx_grad.
+// Volume kernel: flux and f~ = S F in FP64, then per line the jump F^C - n~ . f~,
+// divergence and correction in fixed point; R = -div / J and the RK epilogue
+// in FP64, the next stage's u_f by lines in fixed point.  visc: the viscous
+// flux of k_hexfx_grad; AA: f~ comes projected in tflux.
 template <int N, int EPB, bool NS, bool AA = false>
 __global__ void __launch_bounds__(EPB* FxGeom<N>::TPE, N == 3 ? 2 : 3)
     k_hexfx_vol(long long ne, const double* __restrict__ u, const double* __restrict__ visc,
-                const double* __restrict__ fc, const FxCoef* __restrict__ sq,
-                const int* __restrict__ sex, const double* __restrict__ rcpdjac,
-                const __grid_constant__ HexFxOps op, Phys<double> ph,
-                HexStage<double, double> sa, const double* __restrict__ tflux = nullptr) {
+                const double* __restrict__ fc, const double* __restrict__ smat,
+                const double* __restrict__ rcpdjac, const __grid_constant__ HexFxOps op,
+                Phys<double> ph, HexStage<double, double> sa,
+                const double* __restrict__ tflux = nullptr) {
   using G = FxGeom<N>;
   constexpr int NU = G::NU, NF = G::NF, N2 = G::N2, TPE = G::TPE, PN = G::PN;
-  constexpr int NFT = (NF + TPE - 1) / TPE;
-  constexpr int kGrp[5] = {0, 1, 1, 1, 2};  // exponent group of a variable
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int le = threadIdx.x / TPE, z = threadIdx.x - le * TPE, wz = z >> 5;
+  const int le = threadIdx.x / TPE, z = threadIdx.x - le * TPE;
   const long long e = (long long)blockIdx.x * (blockDim.x / TPE) + le;
   if (e >= ne) return;  // whole elements: their barriers are their own
-  FxCoef* ft = reinterpret_cast<FxCoef*>(smem_raw + le * hexfx_bytes_per_elem<N>(false));
-  FxCoef* jm = ft + 15 * PN;
-  unsigned* ex = reinterpret_cast<unsigned*>(jm + 5 * NF);
-  unsigned* es = ex + 6 * G::WPE;  // [5] maxima of the next stage value
+  double* cs = reinterpret_cast<double*>(smem_raw + le * hexfx_bytes_per_elem<N>(false));
+  double* ft = cs + 5 * NF;  // [15][PN]: f~, then divergence terms (integers)
+  unsigned* ml = reinterpret_cast<unsigned*>(ft + 15 * PN);
   const bool pt = z < NU;
   const int a = z % N, b = (z / N) % N, c = z / N2;
   const int slot = G::slot(a, b, c);
-  if (z < 5) es[z] = 0;
-  // exponents of the point fluxes [0..2] and the interface fluxes [3..5] of
-  // the mass, momentum and energy groups; the interface fluxes wait in their
-  // slots (read back by the same thread)
-  unsigned mx[6] = {0, 0, 0, 0, 0, 0};
-#pragma unroll
-  for (int i = 0; i < NFT; ++i) {
-    if (z + i * TPE < NF) {
-#pragma unroll
-      for (int k = 0; k < 5; ++k) {
-        const double x = fc[(e * 5 + k) * NF + z + i * TPE];
-        mx[3 + kGrp[k]] = max(mx[3 + kGrp[k]], fx_mag(x));
-        jm[k * NF + z + i * TPE] = fx_pack(__double_as_longlong(x));
-      }
-    }
-  }
-  // point fluxes: mass and energy [3] each, momentum tensor [6]; AA: the
-  // transformed flux [15]
-  constexpr int NV = AA ? 15 : 12;
-  double f[NV];
-#pragma unroll
-  for (int q = 0; q < NV; ++q) f[q] = 0.0;
+  async_copy(cs, fc + e * 5 * NF, 5 * NF * int(sizeof(double)), z, TPE);
   if (pt) {
+    double* p = ft + slot;
     if constexpr (AA) {
 #pragma unroll
-      for (int q = 0; q < 15; ++q) f[q] = tflux[(e * 15 + q) * NU + z];
+      for (int q = 0; q < 15; ++q) p[q * PN] = tflux[(e * 15 + q) * NU + z];
     } else {
-      double uz[5], tq[9];
+      double uz[5], tq[9], f[12], S[9];
 #pragma unroll
       for (int k = 0; k < 5; ++k) uz[k] = u[(e * 5 + k) * NU + z];
       if (NS) {
 #pragma unroll
         for (int r = 0; r < 9; ++r) tq[r] = visc[(e * 9 + r) * NU + z];
       }
+#pragma unroll
+      for (int r = 0; r < 9; ++r) S[r] = smat[(e * 9 + r) * NU + z];
       flux_point<double, NS>(uz, tq, ph, f);
-    }
-  }
-#pragma unroll
-  for (int q = 0; q < NV; ++q) {
-    const int gq = AA ? kGrp[q % 5] : (q < 3 ? 0 : q < 9 ? 1 : 2);
-    mx[gq] = max(mx[gq], fx_mag(f[q]));
-  }
-  fx_warp_max<6>(mx, ex, wz);
-  FxCoef S[9];
-  int se = 1023;
-  if (!AA) {
-    if (pt) {
-#pragma unroll
-      for (int r = 0; r < 9; ++r) S[r] = sq[(e * 9 + r) * NU + z];
-    }
-    se = sex[e * 4];
-  }
-  fx_sync<G::WPE, EPB>(le);
-  // common exponent of f~ and F^C per group; f~ = S F is below
-  // 3 2^(E_F + E_S) < 2^(E_F + E_S + 2)
-  int ef[3], ev[3], sh[3];
-  bool bad[3], edge = false;
-#pragma unroll
-  for (int q = 0; q < 3; ++q) {
-    ef[q] = max(int(fx_field_max<6, G::WPE>(ex, q) >> 20), kFxMinExp);
-    const int ec = int(fx_field_max<6, G::WPE>(ex, 3 + q) >> 20);
-    const int eft = AA ? ef[q] : ef[q] + se - 1022 + 2;
-    bad[q] = ef[q] >= 2047 || ec >= 2047;
-    ev[q] = max(max(eft, ec), kFxMinExp);
-    sh[q] = min(ev[q] - eft, 63);
-    edge |= bad[q] || fx_edge(ev[q], se);
-  }
-  if (pt) {
-    if constexpr (AA) {
-#pragma unroll
-      for (int q = 0; q < 15; ++q) ft[q * PN + slot] = fx_split(fx_from(f[q], ev[kGrp[q % 5]]));
-    } else {
-      FxCoef F[12];
-#pragma unroll
-      for (int q = 0; q < 12; ++q)
-        F[q] = fx_split(fx_from(f[q], ef[q < 3 ? 0 : q < 9 ? 1 : 2]));
       // row of variable k: the three fluxes F[j][k]
       constexpr int kIdx[5][3] = {{0, 1, 2}, {3, 6, 7}, {6, 4, 8}, {7, 8, 5}, {9, 10, 11}};
 #pragma unroll
       for (int d = 0; d < 3; ++d)
 #pragma unroll
-        for (int k = 0; k < 5; ++k) {
-          FxSum<0> s;
-#pragma unroll
-          for (int j = 0; j < 3; ++j) s.add(S[d * 3 + j], F[kIdx[k][j]]);
-          ft[(d * 5 + k) * PN + slot] = fx_split(s.value() >> sh[kGrp[k]]);
-        }
+        for (int k = 0; k < 5; ++k)
+          p[(d * 5 + k) * PN] = S[d * 3] * f[kIdx[k][0]] + S[d * 3 + 1] * f[kIdx[k][1]] +
+                                S[d * 3 + 2] * f[kIdx[k][2]];
     }
   }
-#pragma unroll
-  for (int i = 0; i < NFT; ++i)
-#pragma unroll
-    for (int k = 0; k < 5; ++k)
-      if (z + i * TPE < NF) {
-        FxCoef* p = jm + k * NF + z + i * TPE;
-        *p = fx_split(fx_from(__longlong_as_double(fx_unpack(*p)), ev[kGrp[k]]));
-      }
+  cp_async_wait_all();
   fx_sync<G::WPE, EPB>(le);
-  // lines: jump F^C - n~ . f~ at the two faces (scale 2^sm above the field's,
+  // lines: jump F^C - n~ . f~ at the two faces (scale 2^sm above the line's,
   // |jump| <= 1.5 2^59; times -1 on the minus face), then the N divergence
   // terms, in place of the line's own f~ values
   for (int t = z; t < 15 * N2; t += TPE) {
     const int k = t / (3 * N2), r = t - k * 3 * N2, d = r / N2, l = r - d * N2;
     int s0, st, fm;
     fx_line<N>(d, l, &s0, &st, &fm);
-    FxCoef* p = ft + (d * 5 + k) * PN + s0;
-    FxPairs<N> v;
-    v.load(p, st);
+    double* p = ft + (d * 5 + k) * PN + s0;
+    const double c0 = cs[k * NF + fm], c1 = cs[k * NF + fm + N2];
+    double v[N];
+    const unsigned mag = fx_load<N>(p, st, v, max(fx_mag(c0), fx_mag(c1)));
+    const int em = fx_exp(mag);
+    FxPairs<N> w;
+    w.set(v, em);
     long long f0, f1, o[N];
-    v.faces(op, &f0, &f1);
-    const long long cm = fx_join(jm[k * NF + fm]), cp = fx_join(jm[k * NF + fm + N2]);
-    const FxCoef j0 = fx_split(-((cm >> op.sm) + f0));
-    const FxCoef j1 = fx_split((cp >> op.sm) - f1);
-    v.template derivative<2>(op.v, j0, j1, o);
+    w.faces(op, &f0, &f1);
+    const FxCoef j0 = fx_split(-((fx_join(fx_limbs(c0, em)) >> op.sm) + f0));
+    const FxCoef j1 = fx_split((fx_join(fx_limbs(c1, em)) >> op.sm) - f1);
+    w.template derivative<2>(op.v, j0, j1, o);
 #pragma unroll
-    for (int i = 0; i < N; ++i) p[i * st] = fx_pack(o[i]);
+    for (int i = 0; i < N; ++i) p[i * st] = __longlong_as_double(o[i]);
+    ml[(d * 5 + k) * N2 + l] = mag;
   }
   fx_sync<G::WPE, EPB>(le);
   double s[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
@@ -667,45 +481,34 @@ __global__ void __launch_bounds__(EPB* FxGeom<N>::TPE, N == 3 ? 2 : 3)
     const int b0 = op.sv - 1022 - 61 + 1023;
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
-      const long long dv = fx_unpack(ft[k * PN + slot]) + fx_unpack(ft[(5 + k) * PN + slot]) +
-                           fx_unpack(ft[(10 + k) * PN + slot]);
-      const int q = kGrp[k];
-      R[k] = fx_to(dv, ev[q] + b0);
-      if (edge) R[k] = fx_to_edge(dv, ev[q] + b0, bad[q]);
+      // the point's lines of the three directions, in units of the largest
+      const unsigned m0 = ml[k * N2 + b + N * c], m1 = ml[(5 + k) * N2 + a + N * c],
+                     m2 = ml[(10 + k) * N2 + a + N * b];
+      const unsigned mag = max(m0, max(m1, m2));
+      const int em = fx_exp(mag);
+      const long long dv = (__double_as_longlong(ft[k * PN + slot]) >> min(em - fx_exp(m0), 63)) +
+                           (__double_as_longlong(ft[(5 + k) * PN + slot]) >> min(em - fx_exp(m1), 63)) +
+                           (__double_as_longlong(ft[(10 + k) * PN + slot]) >> min(em - fx_exp(m2), 63));
+      R[k] = fx_to(dv, em + b0);
+      if (fx_edge(mag)) R[k] = fx_to_edge(dv, em + b0, mag);
       R[k] = -R[k] * rj;
     }
     // (the point's u serves bare right-hand sides' unused next value only)
     hex_stage_apply(sa, e * 5 * NU + z, NU, s, R, xr, ar, s);
+#pragma unroll
+    for (int k = 0; k < 5; ++k) ft[k * PN + slot] = s[k];
   }
   if (sa.uf_next == nullptr) return;
-  unsigned ms[5];
-#pragma unroll
-  for (int k = 0; k < 5; ++k) ms[k] = fx_mag(s[k]);
-  fx_max_to<5>(ms, es);
-  fx_sync<G::WPE, EPB>(le);
-  if (pt) {
-#pragma unroll
-    for (int k = 0; k < 5; ++k)
-      ft[k * PN + slot] = fx_split(fx_from(s[k], max(int(es[k] >> 20), kFxMinExp)));
-  }
   fx_sync<G::WPE, EPB>(le);
   for (int t = z; t < 15 * N2; t += TPE) {
     const int k = t / (3 * N2), r = t - k * 3 * N2, d = r / N2, l = r - d * N2;
     int s0, st, fm;
     fx_line<N>(d, l, &s0, &st, &fm);
-    FxPairs<N> v;
-    v.load(ft + k * PN + s0, st);
-    long long f0, f1;
-    v.faces(op, &f0, &f1);
-    const int em = max(int(es[k] >> 20), kFxMinExp), bx = em - 1022 + op.sm - 59 + 1023;
-    double v0 = fx_to(f0, bx), v1 = fx_to(f1, bx);
-    if (fx_edge(em)) {
-      v0 = fx_to_edge(f0, bx, em >= 2047);
-      v1 = fx_to_edge(f1, bx, em >= 2047);
-    }
     double* o = sa.uf_next + (e * 5 + k) * NF + fm;
-    o[0] = v0;
-    o[N2] = v1;
+    double f0, f1;
+    fx_faces<N>(op, ft + k * PN + s0, st, &f0, &f1);
+    o[0] = f0;
+    o[N2] = f1;
   }
 }
 

@@ -116,12 +116,7 @@ struct DevType {
   void* NREF = nullptr;
   HexOps<double> hx64{};
   HexOps<float> hx32{};
-  // FP64 fixed-point kernels: line operators, S and S / det J in limbs
-  // [ne][9][nu], their exponents [ne][4]
-  HexFxOps hxfx{};
-  FxCoef* fxs = nullptr;
-  FxCoef* fxj = nullptr;
-  int* fxe = nullptr;
+  HexFxOps hxfx{};          // line operators of the FP64 fixed-point kernels
   // entropy filter (allocated by fr_filter_enable)
   void* fVinvT = nullptr;
   void* fVT = nullptr;
@@ -910,22 +905,7 @@ int setup_device(fr_mesh* m) {
     if (D.kind == EK_HEX) {
       D.hx64 = hex_ops<double>(R);
       D.hx32 = hex_ops<float>(R);
-      if constexpr (sizeof(T) == 8) {
-        if (m->order >= 2) {
-          D.hxfx = hex_fx_ops(R);
-          const size_t bytes = size_t(D.ne) * 9 * D.nu * sizeof(FxCoef);
-          if ((rc = dev_zeros(m, bytes, (void**)&D.fxs))) return rc;
-          if (m->physics == FR_NAVIER_STOKES && (rc = dev_zeros(m, bytes, (void**)&D.fxj)))
-            return rc;
-          if ((rc = dev_zeros(m, size_t(D.ne) * 4 * sizeof(int), (void**)&D.fxe))) return rc;
-          dispatch(D.kind, m->order, [&](auto nu, auto) {
-            k_fx_metric<decltype(nu)::value><<<unsigned((D.ne * 32 + 255) / 256), 256>>>(
-                D.ne, (const double*)D.smat, (const double*)D.rcpdjac, D.fxs, D.fxj, D.fxe);
-          });
-          CK(cudaGetLastError());
-          CK(cudaDeviceSynchronize());
-        }
-      }
+      if (sizeof(T) == 8 && m->order >= 2) D.hxfx = hex_fx_ops(R);
       if (sizeof(T) == 4 && !D.curved) {  // vertex metrics for the FP32-value kernels
         std::vector<double> xv(size_t(D.ne) * 24);
         for (long long e = 0; e < D.ne; ++e)
@@ -1540,9 +1520,6 @@ inline DevType sub_view(const fr_mesh* m, const DevType& D, long long e0, long l
   V.R = sh(D.R, 5 * nu * w);
   V.smat = sh(D.smat, 9 * nu * w);
   V.rcpdjac = sh(D.rcpdjac, nu * w);
-  V.fxs = static_cast<FxCoef*>(sh(D.fxs, 9 * nu * sizeof(FxCoef)));
-  V.fxj = static_cast<FxCoef*>(sh(D.fxj, 9 * nu * sizeof(FxCoef)));
-  V.fxe = static_cast<int*>(sh(D.fxe, 4 * sizeof(int)));
   // [ne][9][nu] where the kernels store the viscous flux: a range's start is
   // the whole type's, since a stage's phases may run over different ranges
   V.grad = sh(D.grad, (stores_visc(m, D) ? 9 : 15) * nu * w);
@@ -1674,11 +1651,13 @@ void launch_stage(fr_mesh* m, cudaStream_t s, int mode, int stage,
             const size_t sm = size_t(eb) * hexfx_bytes_per_elem<N>(true);
             const T* uin = from_x ? (const T*)D.X : (const T*)D.Y;
             if (m->aa_qdeg > 0)
-              k_hexfx_grad<N, E, true><<<grid, tpb, sm, s>>>(D.ne, uin, ta, D.fxj, D.fxe, D.hxfx,
-                                                             ph, (T*)D.grad, va.q);
+              k_hexfx_grad<N, E, true><<<grid, tpb, sm, s>>>(
+                  D.ne, uin, ta, (const T*)D.smat, (const T*)D.rcpdjac, D.hxfx, ph, (T*)D.grad,
+                  va.q);
             else
-              k_hexfx_grad<N, E, false><<<grid, tpb, sm, s>>>(D.ne, uin, ta, D.fxj, D.fxe, D.hxfx,
-                                                              ph, (T*)D.grad, va.q);
+              k_hexfx_grad<N, E, false><<<grid, tpb, sm, s>>>(
+                  D.ne, uin, ta, (const T*)D.smat, (const T*)D.rcpdjac, D.hxfx, ph, (T*)D.grad,
+                  va.q);
           } else {
             const unsigned grid = nblk(D.ne, eb), tpb = hexl_threads<N>(eb);
             const size_t sm = size_t(eb) * hexl_grad_bytes<T, N>();
@@ -1800,15 +1779,15 @@ void launch_stage(fr_mesh* m, cudaStream_t s, int mode, int stage,
           const T* uin = from_x ? (const T*)D.X : (const T*)D.Y;
           if (aa)
             k_hexfx_vol<N, E, false, true><<<grid, tpb, sm, s>>>(
-                D.ne, uin, nullptr, fc, nullptr, nullptr, (const T*)D.rcpdjac, D.hxfx, ph, sa,
+                D.ne, uin, nullptr, fc, nullptr, (const T*)D.rcpdjac, D.hxfx, ph, sa,
                 (const T*)D.tf);
           else if (ns)
             k_hexfx_vol<N, E, true><<<grid, tpb, sm, s>>>(
-                D.ne, uin, (const T*)D.grad, fc, D.fxs, D.fxe, (const T*)D.rcpdjac,
+                D.ne, uin, (const T*)D.grad, fc, (const T*)D.smat, (const T*)D.rcpdjac,
                 D.hxfx, ph, sa);
           else
             k_hexfx_vol<N, E, false><<<grid, tpb, sm, s>>>(
-                D.ne, uin, nullptr, fc, D.fxs, D.fxe, (const T*)D.rcpdjac, D.hxfx, ph, sa);
+                D.ne, uin, nullptr, fc, (const T*)D.smat, (const T*)D.rcpdjac, D.hxfx, ph, sa);
         } else {
           const size_t sm = size_t(eb) * hexl_vol_bytes<T, N>();
           const unsigned grid = nblk(D.ne, eb), tpb = hexl_threads<N>(eb);
