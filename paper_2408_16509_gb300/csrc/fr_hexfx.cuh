@@ -67,6 +67,8 @@ struct HexFxOps {
   HexFxLine g, v;        // gradient; volume (the jump's scale folded in)
   FxCoef ie[3], io[2];
   int sg, sv, sm;        // row scales (powers of two) of g, v and ie / io
+  int gather;            // 1: Gauss-Lobatto lines, the face points are the line
+                         //    end points
 };
 
 // orders that have the fixed-point kernels (p = 1 keeps the FP64 lines: its
@@ -250,12 +252,17 @@ __device__ __forceinline__ unsigned fx_load(const double* p, int st, double (&v)
   return mag;
 }
 
-// values at a line's two faces
+// values at a line's two faces (Gauss-Lobatto: the line's end points)
 template <int N>
 __device__ __forceinline__ void fx_faces(const HexFxOps& op, const double* p, int st, double* f0,
                                          double* f1) {
   double v[N];
   const unsigned mag = fx_load<N>(p, st, v);
+  if (op.gather) {
+    *f0 = v[0];
+    *f1 = v[N - 1];
+    return;
+  }
   const int em = fx_exp(mag), bx = em - 1022 + op.sm - 59 + 1023;
   FxPairs<N> w;
   long long r0, r1;

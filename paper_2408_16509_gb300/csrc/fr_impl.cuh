@@ -622,6 +622,7 @@ inline HexFxOps hex_fx_ops(const RefElement& R) {
     o.io[m] = limbs(DD(0.5) * (X.lm[m] - X.lm[n - 1 - m]), o.sm);
   }
   if (n % 2) o.ie[P] = limbs(X.lm[P], o.sm);
+  o.gather = R.family == 1;
   return o;
 }
 
