@@ -32,24 +32,25 @@ template <>
 __device__ __forceinline__ float fr_sqrt<float>(float x) { return sqrtf(x); }
 
 // Rusanov flux along n.  Both sides' inviscid fluxes are added before the
-// halving and the velocity components are never formed (n.m and m.m of the
-// momentum m serve the flux, the pressure and the wave speed): 89 FP64
-// instructions a pair with the two reciprocals and roots, 100 with one flux
-// per side.
+// halving (one flux per side: 7 FP64 instructions a pair more).  Products are
+// of a momentum and a velocity: the momenta's squares leave the type's range at
+// states of 1e19 or 1e-19 in FP32, and were slower (interface kernel, FP64-pipe
+// bound, 24^3 p = 4: 447 us against 430).
 template <typename T>
 __device__ __forceinline__ void rusanov(const T ul[5], const T ur[5],
                                         const T n[3], const Phys<T>& ph,
                                         T F[5]) {
   const T il = T(1) / ul[0], ir = T(1) / ur[0];
-  const T ml = ul[1] * n[0] + ul[2] * n[1] + ul[3] * n[2];
-  const T mr = ur[1] * n[0] + ur[2] * n[1] + ur[3] * n[2];
-  const T vl = ml * il, vr = mr * ir;
-  const T pl = ph.gm1 * (ul[4] - (T(0.5) * il) * (ul[1] * ul[1] + ul[2] * ul[2] + ul[3] * ul[3]));
-  const T pr = ph.gm1 * (ur[4] - (T(0.5) * ir) * (ur[1] * ur[1] + ur[2] * ur[2] + ur[3] * ur[3]));
+  const T wl[3] = {ul[1] * il, ul[2] * il, ul[3] * il};
+  const T wr[3] = {ur[1] * ir, ur[2] * ir, ur[3] * ir};
+  const T vl = wl[0] * n[0] + wl[1] * n[1] + wl[2] * n[2];
+  const T vr = wr[0] * n[0] + wr[1] * n[1] + wr[2] * n[2];
+  const T pl = ph.gm1 * (ul[4] - T(0.5) * (ul[1] * wl[0] + ul[2] * wl[1] + ul[3] * wl[2]));
+  const T pr = ph.gm1 * (ur[4] - T(0.5) * (ur[1] * wr[0] + ur[2] * wr[1] + ur[3] * wr[2]));
   const T a = fabs(vl) + fr_sqrt<T>(ph.gamma * pl * il);
   const T b = fabs(vr) + fr_sqrt<T>(ph.gamma * pr * ir);
   const T hl = T(0.5) * (a > b ? a : b), ps = pl + pr;
-  F[0] = T(0.5) * (ml + mr) + hl * (ul[0] - ur[0]);
+  F[0] = T(0.5) * (ul[0] * vl + ur[0] * vr) + hl * (ul[0] - ur[0]);
 #pragma unroll
   for (int k = 0; k < 3; ++k)
     F[1 + k] = T(0.5) * (ul[1 + k] * vl + ur[1 + k] * vr + ps * n[k]) + hl * (ul[1 + k] - ur[1 + k]);
@@ -164,7 +165,7 @@ __device__ __forceinline__ void flux_point(const T u[5], const T tq[9], const Ph
 // - 2/3 n_i (div m - v.grad rho), (tau n)_i = (mu / rho) x_i, energy
 // (mu / rho) v.x + (kappa / rho) rho n.grad e.  The velocity gradient is
 // never built: 59 instructions a side against 75 (interface kernel, FP64-pipe
-// bound, 24^3 p = 4: 485 -> 447 us with the Rusanov form above).
+// bound, 24^3 p = 4: 485 -> 430 us with the Rusanov form above).
 // FP32: (tau n)_i = mu (sum_j (dv_i/dx_j + dv_j/dx_i) n_j - 2/3 div v n_i) from
 // the velocity gradient; the form above made the prism and tetrahedron
 // gradient kernels 1 % slower.
