@@ -2296,37 +2296,42 @@ int resolve_variant(fr_mesh* m, int scheme, double dt) {
     // step replayed: launched one by one, a small mesh's step is bound by the
     // launches and the choice was noise (11 x 9 x 7 cells of mixed elements,
     // FP64 p = 2: types on parallel branches were kept in about half of the
-    // runs, 0.97 ms a step replayed against 0.72 in order).
+    // runs, 0.97 ms a step replayed against 0.72 in order).  On a stream that
+    // cannot be captured (the legacy default stream) steps are launched one by
+    // one, so they are timed like that.
     auto replay = [&](float* ms) -> int {
+      if (cudaStreamBeginCapture(m->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
+        cudaGetLastError();
+        return run(nullptr, ms);
+      }
+      for (int s2 = 0; s2 < nst; ++s2) launch_stage<T, TR>(m, m->stream, mode, s2);
       cudaGraph_t g = nullptr;
       cudaGraphExec_t ge = nullptr;
-      CK(cudaStreamBeginCapture(m->stream, cudaStreamCaptureModeThreadLocal));
-      for (int s2 = 0; s2 < nst; ++s2) launch_stage<T, TR>(m, m->stream, mode, s2);
-      CK(cudaStreamEndCapture(m->stream, &g));
-      cudaError_t err = cudaGraphInstantiate(&ge, g, 0);
-      cudaGraphDestroy(g);
-      if (err != cudaSuccess)
-        return fail(FR_ECUDA, std::string("autotuner: ") + cudaGetErrorString(err));
+      cudaError_t err = cudaStreamEndCapture(m->stream, &g);
+      if (err == cudaSuccess) err = cudaGraphInstantiate(&ge, g, 0);
+      if (g) cudaGraphDestroy(g);
+      int rr = FR_OK;
       *ms = 1e30f;
-      for (int rep = 0; rep < 3; ++rep) {  // the first one untimed
+      for (int rep = 0; rep < 3 && err == cudaSuccess && rr == FR_OK; ++rep) {  // 0: untimed
         for (size_t t = 0; t < nt; ++t)
           cudaMemcpyAsync(m->types[t].X, saved[t],
                           size_t(m->types[t].ne) * 5 * m->types[t].nu * sizeof(TR),
                           cudaMemcpyDeviceToDevice, m->stream);
         m->uf_valid = false;
-        ensure_uf<T, TR>(m);
+        rr = ensure_uf<T, TR>(m);
         cudaEventRecord(e0, m->stream);
-        cudaGraphLaunch(ge, m->stream);
+        err = cudaGraphLaunch(ge, m->stream);
         cudaEventRecord(e1, m->stream);
-        err = cudaStreamSynchronize(m->stream);
+        const cudaError_t es = cudaStreamSynchronize(m->stream);
+        if (err == cudaSuccess) err = es;
         float t = 0.f;
-        cudaEventElapsedTime(&t, e0, e1);
+        if (err == cudaSuccess) err = cudaEventElapsedTime(&t, e0, e1);
         if (rep > 0) *ms = std::min(*ms, t);
       }
-      cudaGraphExecDestroy(ge);
-      if (err != cudaSuccess)
-        return fail(FR_ECUDA, std::string("autotuner: ") + cudaGetErrorString(err));
-      return FR_OK;
+      if (ge) cudaGraphExecDestroy(ge);
+      if (rr == FR_OK && err != cudaSuccess)
+        rr = fail(FR_ECUDA, std::string("autotuner: ") + cudaGetErrorString(err));
+      return rr;
     };
     float bt = 1e30f;
     int btb = 256;
