@@ -9,7 +9,7 @@ int setup_filter(fr_mesh* m) {
   int rc;
   for (size_t t = 0; t < m->types.size(); ++t) {
     DevType& D = m->types[t];
-    if (D.fVT) continue;
+    if (D.filter_ready) continue;  // (not after a call that failed half-way)
     const RefElement& R = m->host[t].ref;
     const int nu = D.nu, nf = D.nf, np = nu + nf;
     std::vector<double> vinvt(size_t(nu) * nu), vt(size_t(nu) * np), deg(nu);
@@ -36,6 +36,7 @@ int setup_filter(fr_mesh* m) {
     if (sizeof(T) == 4 &&
         (rc = dev_zeros(m, size_t(D.ne) * sizeof(CheckRec), &D.frec)))
       return rc;
+    D.filter_ready = true;
   }
   if ((rc = setup_partner(m))) return rc;
   if (!m->d_fstats) {

@@ -118,6 +118,7 @@ struct DevType {
   HexOps<float> hx32{};
   HexFxOps hxfx{};          // line operators of the FP64 fixed-point kernels
   // entropy filter (allocated by fr_filter_enable)
+  bool filter_ready = false;  // all of them are there
   void* fVinvT = nullptr;
   void* fVT = nullptr;
   void* fdeg = nullptr;
@@ -282,6 +283,7 @@ struct fr_mesh {
   // parallel branches (streams forked and joined inside the captured graph)
   int face_tb = 256;
   bool par_types = false;
+  bool partner_ready = false;  // every type's fpartner is filled
   std::vector<cudaStream_t> par_st;
   std::vector<cudaEvent_t> par_ev;
   float sched_ms[2] = {0.f, 0.f};  // step time before / after tile tuning
@@ -746,14 +748,16 @@ static __global__ void k_partner(int np, const int32_t* __restrict__ pl,
 }
 
 inline int setup_partner(fr_mesh* m) {
+  if (m->partner_ready) return FR_OK;
   int32_t* p[3] = {nullptr, nullptr, nullptr};
   int nf[3] = {1, 1, 1};
   for (size_t t = 0; t < m->types.size(); ++t) {
     DevType& D = m->types[t];
-    if (D.fpartner) return FR_OK;
     const size_t bytes = size_t(D.ne) * D.nf * sizeof(int32_t);
-    CK(cudaMalloc((void**)&D.fpartner, bytes));
-    m->allocs.push_back(D.fpartner);
+    if (!D.fpartner) {  // (there already after a call that failed at a later type)
+      CK(cudaMalloc((void**)&D.fpartner, bytes));
+      m->allocs.push_back(D.fpartner);
+    }
     CK(cudaMemset(D.fpartner, 0xff, bytes));
     p[t] = D.fpartner;
     nf[t] = D.nf;
@@ -763,6 +767,7 @@ inline int setup_partner(fr_mesh* m) {
                                                        nf[0], nf[1], nf[2]);
   CK(cudaGetLastError());
   CK(cudaDeviceSynchronize());
+  m->partner_ready = true;
   return FR_OK;
 }
 
