@@ -195,12 +195,6 @@ __device__ __forceinline__ double pressure64(const double v[5], double g) {
   return (g - 1.0) * (v[4] - 0.5 * (v[1] * v[1] + v[2] * v[2] + v[3] * v[3]) / v[0]);
 }
 
-__device__ __forceinline__ double warp_min(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmin(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
-
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -482,18 +476,6 @@ static __global__ void k_entropy_value(long long ne, const EntropyRec* __restric
   smin[e] = isfinite(m) ? m : 0.0;
 }
 
-// Block-wide reductions for the filter kernel.
-__device__ __forceinline__ double block_min(double v, double* red) {
-  v = warp_min(v);
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __syncthreads();
-  if (lane == 0) red[w] = v;
-  __syncthreads();
-  double r = INFINITY;
-  for (int i = 0; i < kFilterThreads / 32; ++i) r = fmin(r, red[i]);
-  return r;
-}
-
 // Order-preserving integer key of a double (signed compare of keys = fmin
 // order, positive NaN last), so that minima of doubles reduce on the
 // integer pipes instead of the (slow) FP64 pipe.
@@ -504,35 +486,6 @@ __device__ __forceinline__ long long dkey(double x) {
 
 __device__ __forceinline__ double dunkey(long long k) {
   return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffLL));
-}
-
-// exact minima of three doubles over the block (one pair of barriers)
-__device__ __forceinline__ void block_min3_key(double& a, double& b, double& c,
-                                               long long* red) {
-  long long ka = dkey(a), kb = dkey(b), kc = dkey(c);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    ka = min(ka, __shfl_xor_sync(0xffffffffu, ka, o));
-    kb = min(kb, __shfl_xor_sync(0xffffffffu, kb, o));
-    kc = min(kc, __shfl_xor_sync(0xffffffffu, kc, o));
-  }
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __syncthreads();
-  if (lane == 0) {
-    red[3 * w] = ka;
-    red[3 * w + 1] = kb;
-    red[3 * w + 2] = kc;
-  }
-  __syncthreads();
-  ka = kb = kc = 0x7fffffffffffffffLL;
-  for (int i = 0; i < kFilterThreads / 32; ++i) {
-    ka = min(ka, red[3 * i]);
-    kb = min(kb, red[3 * i + 1]);
-    kc = min(kc, red[3 * i + 2]);
-  }
-  a = dunkey(ka);
-  b = dunkey(kb);
-  c = dunkey(kc);
 }
 
 // minima of four integer keys over the block (one pair of barriers)

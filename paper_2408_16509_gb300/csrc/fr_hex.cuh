@@ -232,16 +232,6 @@ __device__ __forceinline__ void hex_stage_load(const HexStage<T, TR>& a,
   }
 }
 
-template <typename T, typename TR>
-__device__ __forceinline__ void hex_stage_update(const HexStage<T, TR>& a,
-                                                 long long i0, long long vstr,
-                                                 const T u[5], const T R[5],
-                                                 T s[5]) {
-  TR x[5], ac[5];
-  hex_stage_load(a, i0, vstr, x, ac);
-  hex_stage_apply(a, i0, vstr, u, R, x, ac, s);
-}
-
 // interpolate smem field src[v][pt] to face point fp (5 variables)
 template <typename T, int N, int NV, typename Ops>
 __device__ __forceinline__ void face_interp(const T* src, int fp, const Ops& op,
@@ -264,38 +254,6 @@ __device__ __forceinline__ void face_interp(const T* src, int fp, const Ops& op,
     T c = w[m];
 #pragma unroll
     for (int k = 0; k < NV; ++k) out[k] += c * src[k * N * N * N + q];
-  }
-}
-
-// Both faces of direction dir at face position (i, j): their flux points
-// lie on the same line of solution points, so one pass over the line's N
-// points (shared-memory reads) gives both values (o0: minus face, o1: plus
-// face) with the weights l_m(-1), l_m(+1).
-template <typename T, int N, int NV, typename Ops>
-__device__ __forceinline__ void face_interp_pair(const T* src, int dir, int i, int j,
-                                                 const Ops& op, T o0[NV], T o1[NV]) {
-  constexpr int NU = N * N * N;
-  if (op.gather) {  // Gauss-Lobatto: the line's end points
-    const int q0 = line_pt<N>(2 * dir, i, j, 0), q1 = line_pt<N>(2 * dir, i, j, N - 1);
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      o0[k] = src[k * NU + q0];
-      o1[k] = src[k * NU + q1];
-    }
-    return;
-  }
-#pragma unroll
-  for (int k = 0; k < NV; ++k) o0[k] = o1[k] = T(0);
-#pragma unroll
-  for (int m = 0; m < N; ++m) {
-    const int q = line_pt<N>(2 * dir, i, j, m);
-    const T cm = op.lm[m], cp = op.lp[m];
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      const T v = src[k * NU + q];
-      o0[k] += cm * v;
-      o1[k] += cp * v;
-    }
   }
 }
 

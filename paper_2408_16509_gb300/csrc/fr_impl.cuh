@@ -137,10 +137,9 @@ struct DevType {
   int pri_nm = 0, pri_nl = 0;
   void* pri_img = nullptr;
   int pri_grad_ctas = 1, pri_vol_ctas = 1;
-  // tetrahedra and prisms, FP32 values: operators of fr_simplex.cuh for the
-  // gradient and the volume kernel
+  // tetrahedra and prisms, FP32 values: operators of fr_simplex.cuh
   bool sx_ok = false;
-  SimplexOps sx_grad{}, sx_vol{};
+  SimplexOps sx{};
   int sx_grad_ctas = 1, sx_vol_ctas = 1;
   // tetrahedra: M0 by its nonzeros (every flux point is a solution point)
   int32_t* m0c = nullptr;
@@ -869,21 +868,17 @@ int setup_device(fr_mesh* m) {
       }
     }
     if (sizeof(T) == 4 && D.kind != EK_HEX) {
-      std::vector<uint32_t> gi, vi;
+      std::vector<uint32_t> sxi;
       dispatch(D.kind, m->order, [&](auto nu, auto nf) {
         constexpr int NU = decltype(nu)::value, NF = decltype(nf)::value;
-        if constexpr (simplex_zb<NU, NF>(true) > 0)
-          D.sx_ok = build_simplex_ops<NU, NF>(R, simplex_zb<NU, NF>(true), gi, D.sx_grad) &&
-                    build_simplex_ops<NU, NF>(R, simplex_zb<NU, NF>(false), vi, D.sx_vol);
+        if constexpr (simplex_zb<NU, NF>() > 0)
+          D.sx_ok = build_simplex_ops<NU, NF>(R, simplex_zb<NU, NF>(), sxi, D.sx);
       });
       if (D.sx_ok) {
-        void *gd = nullptr, *vd = nullptr;
-        if ((rc = dev_zeros(m, gi.size() * 4, &gd)) || (rc = dev_zeros(m, vi.size() * 4, &vd)))
-          return rc;
-        CK(cudaMemcpy(gd, gi.data(), gi.size() * 4, cudaMemcpyHostToDevice));
-        CK(cudaMemcpy(vd, vi.data(), vi.size() * 4, cudaMemcpyHostToDevice));
-        D.sx_grad.img = static_cast<const float*>(gd);
-        D.sx_vol.img = static_cast<const float*>(vd);
+        void* dev = nullptr;
+        if ((rc = dev_zeros(m, sxi.size() * 4, &dev))) return rc;
+        CK(cudaMemcpy(dev, sxi.data(), sxi.size() * 4, cudaMemcpyHostToDevice));
+        D.sx.img = static_cast<const float*>(dev);
         D.pri_ok = D.kind == EK_PRI;
       }
       bool fits = false;
@@ -1108,8 +1103,7 @@ int simplex_eb(long long ne, int num_sms) {
 template <int NU, int NF>
 size_t simplex_smem(const DevType& D, int eb, bool grad) {
   using G = SimplexGeom<NU, NF>;
-  const int nm = (grad ? D.sx_grad : D.sx_vol).nm;
-  return size_t(G::words(simplex_zb<NU, NF>(grad), nm) + eb * (grad ? G::kGrad : G::kVol)) * 4;
+  return size_t(G::words(simplex_zb<NU, NF>(), D.sx.nm) + eb * (grad ? G::kGrad : G::kVol)) * 4;
 }
 
 // their launch: grid and shared memory for the type's tile (CTAs per SM)
@@ -1335,15 +1329,15 @@ int prepare_kernels(fr_mesh* m) {
           D.pri_vol_ctas = pb > 0 ? pb : 1;
         }
       }
-      if constexpr (sizeof(T) == 4 && sizeof(TR) == 4 && simplex_zb<NU, NF>(true) > 0) {
+      if constexpr (sizeof(T) == 4 && sizeof(TR) == 4 && simplex_zb<NU, NF>() > 0) {
         if (D.sx_ok) {
-          constexpr int ZG = simplex_zb<NU, NF>(true), ZV = simplex_zb<NU, NF>(false);
+          constexpr int ZB = simplex_zb<NU, NF>();
           const int eb = simplex_threads<NU>() / NU, th = simplex_threads<NU>();
           const int smg = int(simplex_smem<NU, NF>(D, eb, true));
           const int smv = int(simplex_smem<NU, NF>(D, eb, false));
-          auto xg = k_simplex_grad<NU, NF, ZG>;
-          auto xv0 = k_simplex_vol<NU, NF, ZV, false>;
-          auto xv1 = k_simplex_vol<NU, NF, ZV, true>;
+          auto xg = k_simplex_grad<NU, NF, ZB>;
+          auto xv0 = k_simplex_vol<NU, NF, ZB, false>;
+          auto xv1 = k_simplex_vol<NU, NF, ZB, true>;
           cudaFuncSetAttribute(xg, cudaFuncAttributeMaxDynamicSharedMemorySize, smg);
           cudaFuncSetAttribute(xv0, cudaFuncAttributeMaxDynamicSharedMemorySize, smv);
           cudaFuncSetAttribute(xv1, cudaFuncAttributeMaxDynamicSharedMemorySize, smv);
@@ -1683,15 +1677,15 @@ void launch_stage(fr_mesh* m, cudaStream_t s, int mode, int stage,
       } else if (use_simplex(m, D)) {
         dispatch(D.kind, m->order, [&](auto nu, auto nf) {
           constexpr int NU = decltype(nu)::value, NF = decltype(nf)::value;
-          if constexpr (sizeof(T) == 4 && sizeof(TR) == 4 && simplex_zb<NU, NF>(true) > 0) {
-            constexpr int ZB = simplex_zb<NU, NF>(true);
+          if constexpr (sizeof(T) == 4 && sizeof(TR) == 4 && simplex_zb<NU, NF>() > 0) {
+            constexpr int ZB = simplex_zb<NU, NF>();
             int eb;
             unsigned grid, th;
             size_t sm;
             simplex_launch<NU, NF>(m, D, true, &eb, &grid, &th, &sm);
             const T* uin = from_x ? (const T*)D.X : (const T*)D.Y;
             k_simplex_grad<NU, NF, ZB><<<grid, th, sm, s>>>(
-                D.ne, eb, uin, ta, (const T*)D.smat, (const T*)D.rcpdjac, D.sx_grad,
+                D.ne, eb, uin, ta, (const T*)D.smat, (const T*)D.rcpdjac, D.sx,
                 (T*)D.grad, va, bc, ph);
           }
         });
@@ -1844,8 +1838,8 @@ void launch_stage(fr_mesh* m, cudaStream_t s, int mode, int stage,
       if (use_simplex(m, D)) {
         dispatch(D.kind, m->order, [&](auto nu, auto nf) {
           constexpr int NU = decltype(nu)::value, NF = decltype(nf)::value;
-          if constexpr (sizeof(T) == 4 && sizeof(TR) == 4 && simplex_zb<NU, NF>(false) > 0) {
-            constexpr int ZB = simplex_zb<NU, NF>(false);
+          if constexpr (sizeof(T) == 4 && sizeof(TR) == 4 && simplex_zb<NU, NF>() > 0) {
+            constexpr int ZB = simplex_zb<NU, NF>();
             int eb;
             unsigned grid, th;
             size_t sm;
@@ -1856,10 +1850,10 @@ void launch_stage(fr_mesh* m, cudaStream_t s, int mode, int stage,
             if (ns)
               k_simplex_vol<NU, NF, ZB, true><<<grid, th, sm, s>>>(
                   D.ne, eb, uin, (const T*)D.grad, fc, (const T*)D.smat, (const T*)D.rcpdjac,
-                  D.sx_vol, ph, ha);
+                  D.sx, ph, ha);
             else
               k_simplex_vol<NU, NF, ZB, false><<<grid, th, sm, s>>>(
-                  D.ne, eb, uin, nullptr, fc, (const T*)D.smat, (const T*)D.rcpdjac, D.sx_vol,
+                  D.ne, eb, uin, nullptr, fc, (const T*)D.smat, (const T*)D.rcpdjac, D.sx,
                   ph, ha);
           }
         });

@@ -45,11 +45,11 @@
 namespace frgb {
 
 // threads of a CTA at most: one per point of its elements (eb NU of them) in
-// the point phases.  128 where points nearly fill them (256 took 0-2 % longer at
-// p = 3), else 256.
+// the point phases.  128 where points fill nine tenths of them (256 took 0-2 %
+// longer at p = 3), else 256.
 template <int NU>
 __host__ __device__ constexpr int simplex_threads() {
-  return NU > 25 && NU != 40 ? 256 : 128;
+  return 128 / NU * NU * 10 >= 128 * 9 ? 128 : 256;
 }
 constexpr int kSimplexMaxFaces = 5;
 
@@ -195,8 +195,7 @@ struct SimplexGeom {
 // four; volume 57 and 65; 20480 prisms p = 3: 59 with two, 84 with five).
 // Three divide the triangle points of prisms p = 1, 2.
 template <int NU, int NF>
-constexpr int simplex_zb(bool grad) {
-  (void)grad;
+constexpr int simplex_zb() {
   if (NU == 8 || NU == 27 || NU == 64 || NU == 125) return 0;  // hexahedra
   return NU == 18 || NU == 6 ? 3 : 2;
 }
