@@ -427,7 +427,7 @@ __global__ void __launch_bounds__(EPB* N* N* N)
 #pragma unroll
     for (int i = 0; i < NFT; ++i)
       fb[i] = z + i * NU < NF ? int(va.fbc[e * NF + z + i * NU]) : -1;
-    if (z < 24) xv[z] = verts[e * 24 + z];
+    for (int i = z; i < 24; i += NU) xv[i] = verts[e * 24 + i];  // (p = 1: 8 threads)
   }
   cp_async_wait_all();
   __syncthreads();
@@ -524,7 +524,7 @@ __global__ void __launch_bounds__(EPB* N* N* N)
       uz[k] = uin ? uin[(e * 5 + k) * NU + z] : T(sa.X[(e * 5 + k) * NU + z]);
       us[k * NU + z] = uz[k];
     }
-    if (z < 24) xv[z] = verts[e * 24 + z];
+    for (int i = z; i < 24; i += NU) xv[i] = verts[e * 24 + i];  // (p = 1: 8 threads)
   }
   cp_async_wait_all();
   __syncthreads();
