@@ -85,12 +85,16 @@ constexpr size_t dense_vol_smem(int eb = dense_epb<NU>()) {
           size_t(eb) * size_t(DenseLayout<T, NU, NF>::kVolElem)) * sizeof(T);
 }
 
-// Elements per CTA of those kernels for ne elements: dense_epb, or, when
-// that leaves SMs without a CTA, one group per SM (a warp at least).  756 FP64
-// tetrahedra of order 2 filled 31 CTAs of 25 elements: gradient kernel 63 ->
-// 39 us on 152 CTAs of 5.
-template <int NU>
+// Elements per CTA of those kernels for ne elements: dense_epb, or, with FP64
+// values and when that leaves SMs without a CTA, one group per SM (a warp at
+// least).  756 FP64 tetrahedra of order 2 filled 31 CTAs of 25 elements: gradient
+// kernel 63 -> 39 us on 152 CTAs of 5.  FP32 kernels are short and run beside
+// those of the other types: each CTA's copy of the operators then costs more
+// than idle SMs (anti-aliased FP32 step of 216 tetrahedra, 144 prisms and 108
+// hexahedra of order 3: 266 us so, 235 with dense_epb).
+template <typename T, int NU>
 inline int dense_eb(long long ne, int num_sms) {
+  if (sizeof(T) == 4) return dense_epb<NU>();
   const long long per = (ne + num_sms - 1) / num_sms;
   return int(std::min<long long>(dense_epb<NU>(), std::max<long long>(per, (31 + NU) / NU)));
 }
@@ -1694,7 +1698,7 @@ void launch_stage(fr_mesh* m, cudaStream_t s, int mode, int stage,
           constexpr int NU = decltype(nu)::value, NF = decltype(nf)::value;
           if constexpr (sizeof(T) == 8 && pri_order(NU, NF) > 0) {
             constexpr int E = dense_epb<NU>();
-            const int eb = dense_eb<NU>(D.ne, m->num_sms);
+            const int eb = dense_eb<T, NU>(D.ne, m->num_sms);
             const unsigned grid = unsigned(std::min<long long>(
                 (D.ne + eb - 1) / eb,
                 (long long)m->num_sms * (D.tile_grad > 0 ? D.tile_grad : D.pri_grad_ctas)));
@@ -1708,7 +1712,7 @@ void launch_stage(fr_mesh* m, cudaStream_t s, int mode, int stage,
         dispatch(D.kind, m->order, [&](auto nu, auto nf) {
           constexpr int NU = decltype(nu)::value, NF = decltype(nf)::value;
           constexpr int E = dense_epb<NU>();
-          const int eb = dense_eb<NU>(D.ne, m->num_sms);
+          const int eb = dense_eb<T, NU>(D.ne, m->num_sms);
           const size_t sm = dense_grad_smem<T, NU, NF>(eb);
           const unsigned grid = unsigned(std::min<long long>(
               (D.ne + eb - 1) / eb,
@@ -1862,7 +1866,7 @@ void launch_stage(fr_mesh* m, cudaStream_t s, int mode, int stage,
           constexpr int NU = decltype(nu)::value, NF = decltype(nf)::value;
           if constexpr (sizeof(T) == 8 && pri_order(NU, NF) > 0) {
             constexpr int E = dense_epb<NU>();
-            const int eb = dense_eb<NU>(D.ne, m->num_sms);
+            const int eb = dense_eb<T, NU>(D.ne, m->num_sms);
             const unsigned grid = unsigned(std::min<long long>(
                 (D.ne + eb - 1) / eb,
                 (long long)m->num_sms * (D.tile_vol > 0 ? D.tile_vol : D.pri_vol_ctas)));
@@ -1881,7 +1885,7 @@ void launch_stage(fr_mesh* m, cudaStream_t s, int mode, int stage,
       dispatch(D.kind, m->order, [&](auto nu, auto nf) {
         constexpr int NU = decltype(nu)::value, NF = decltype(nf)::value;
         constexpr int E = dense_epb<NU>();
-        const int eb = dense_eb<NU>(D.ne, m->num_sms);
+        const int eb = dense_eb<T, NU>(D.ne, m->num_sms);
         const size_t sm = dense_vol_smem<T, NU, NF>(eb);
         const unsigned grid = unsigned(std::min<long long>(
             (D.ne + eb - 1) / eb,
