@@ -21,8 +21,8 @@
 // DRAM traffic an element and stage less at p = 4.
 //
 // Measured per launch, 48^3 p = 4 with FP64 registers (32^3 p = 3 FP32):
-// common solution and gradient 155 + 621 -> 586 us (29 + 85 -> 96), volume 657 ->
-// 550-583 us (92 -> 71; 0.9 of its DRAM traffic at the copy rate).  The
+// common solution and gradient 155 + 621 -> 588 us (29 + 85 -> 96), volume 657 ->
+// 560 us (92 -> 71; 0.9 of its DRAM traffic at the copy rate).  The
 // gradient kernel issues on 65 % of the cycles and waits for the traces on
 // most of the others.
 #pragma once
@@ -233,12 +233,21 @@ __global__ void __launch_bounds__(hexl_threads<N>(EPB), sizeof(T) == 4 ? 4 : 2)
   }
 }
 
+// CTAs of the largest tile per SM.  FP32 values: 5 (48 registers); with FP64
+// registers the odd N spill at 48 (100 bytes at N = 5), so 4 there: 24^3 and 48^3
+// p = 4, 95 -> 86 and 669 -> 616 us with the largest tile, 586 -> 560 with the
+// best; N = 4 keeps 5 (48^3: 286, 315 with 4).
+template <typename T, typename TR, int N>
+__host__ __device__ constexpr int hexl_vol_ctas() {
+  return sizeof(T) == 8 ? 2 : sizeof(TR) == 8 && N % 2 ? 4 : 5;
+}
+
 // Volume kernel: f~ = S F at the solution points, then per line the jump
 // F^C - n~ . f~ at its two faces and its N divergence terms (in place of the
 // line's f~), R = -div / J, the RK epilogue and the next stage's u_f.  visc:
 // the viscous flux of k_hexl_grad; AA: f~ comes projected in tflux.
 template <typename T, typename TR, int N, int EPB, bool NS, bool AA = false>
-__global__ void __launch_bounds__(hexl_threads<N>(EPB), sizeof(T) == 4 ? 5 : 2)
+__global__ void __launch_bounds__(hexl_threads<N>(EPB), hexl_vol_ctas<T, TR, N>())
     k_hexl_vol(long long ne, int eb, const T* __restrict__ uin, const T* __restrict__ visc,
                const T* __restrict__ fc, const T* __restrict__ smat,
                const T* __restrict__ rcpdjac, const __grid_constant__ HexOps<T> op, Phys<T> ph,
