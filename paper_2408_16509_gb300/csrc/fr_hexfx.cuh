@@ -36,13 +36,12 @@
 // coefficients.
 //
 // Measured per launch, 24^3 p = 4 (20^3 p = 3) Navier-Stokes: gradient with the
-// solution jumps 850 + 43 -> 427 us (242 + 20 -> 140), volume 1108 -> 292 us
+// solution jumps 850 + 43 -> 427 us (242 + 20 -> 140), volume 1108 -> 291 us
 // (321 -> 94), against FP64 loops with one thread per point; one exponent per
 // element and field and metric products in fixed point took 345 and 269 us
-// (118, 96).  The gradient kernel is bound by the FP64 pipe, some 110
-// instructions a point of 64 clocks a warp; the volume kernel has 90 of them
-// and as much time in integer instructions.  62 to 70 registers; a fourth CTA
-// per SM gained nothing.
+// (118, 96).  Both are bound by the FP64 pipe (82 and 83 % of its rate; integer
+// pipes at 34-38 %): the metric products and the pointwise physics.  62 to 70
+// registers; a fourth CTA per SM gained nothing.
 #pragma once
 #include "fr_hex.cuh"
 

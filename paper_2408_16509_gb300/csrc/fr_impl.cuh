@@ -112,8 +112,8 @@ struct DevType {
   void* R = nullptr;        // right-hand side (fr_rhs)
   void* smat = nullptr;     // [ne][9][nu]
   void* rcpdjac = nullptr;  // [ne][nu]
-  void* grad = nullptr;     // [ne][15][nu] (NS); the FP64 fixed-point kernels
-                            // keep the viscous flux in it, [ne][9][nu]
+  void* grad = nullptr;     // [ne][15][nu] (NS); kernels of stores_visc keep the
+                            // viscous flux in it, [ne][9][nu]
   void* M0T = nullptr;
   void* DT = nullptr;
   void* LIFTT = nullptr;
@@ -1096,7 +1096,7 @@ bool stores_visc(const fr_mesh* m, const DevType& D) {
 }
 
 // elements per CTA of the blocked kernels: a thread per point, fewer where
-// that would leave SMs without a CTA (as dense_eb)
+// that would leave SMs without a CTA (as dense_eb with FP64 values)
 template <int NU>
 int simplex_eb(long long ne, int num_sms) {
   const long long per = (ne + num_sms - 1) / num_sms;

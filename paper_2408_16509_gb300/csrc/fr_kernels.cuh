@@ -671,7 +671,7 @@ __global__ void k_exchange_scatter(int n, const int32_t* __restrict__ list,
 // Dense kernels (prisms, tetrahedra, and the dense hexahedron variant) are
 // persistent: each CTA copies the type's operators into shared memory once
 // (when they fit) and then loops over groups of eb elements (eb NU threads, eb
-// at most EPB; fewer where full groups would leave SMs without any).
+// at most EPB; FP64: fewer where full groups would leave SMs without any).
 
 // one point's row of 5 / 15 values (16-byte aligned rows)
 template <typename T>
